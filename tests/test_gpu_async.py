@@ -229,6 +229,26 @@ def test_mixed_mrca_loaded_matches_oracle(S, b, policy, t_lo, t_hi, n):
     assert np.array_equal(lo, elo), np.nonzero(lo != elo)[0][:5]
 
 
+@pytest.mark.parametrize("n", [2, 31, 32, 33, 63, 64, 65, 97, 129])
+@pytest.mark.parametrize("S,b,policy,t_lo,t_hi", [
+    (64, 1, STEADY, 0, 90), (256, 1, HYBRID, 300, 2000), (4, 8, TILTED, 0, 200), (8, 2, STEADY, 40, 41),
+])
+def test_mixed_mrca_tile_edges(S, b, policy, t_lo, t_hi, n):
+    """Samples around the pair kernel's tile (32 rows x 64 columns) and its warps, for the
+    narrowest and widest surfaces, counters on both sides of the surface's size, empty surfaces
+    (counter 0) and one common counter."""
+    shape = RunShape(rows=4, cols=3, island_size=32, surface_sites=S, differentia_bits=b,
+                     curation=policy, mode=ASYNC)
+    rec = _forked_population(shape.n_agents, S, b, policy, t_lo, t_hi, seed=S + b)
+    g = gpu_run(shape)
+    g.load(rec, 0)
+    ids = np.random.default_rng(n).permutation(shape.n_agents)[:n].astype(np.uint32)
+    lo, hi = g.mrca_bounds(ids)
+    elo, ehi = oracle.mrca_bounds_mixed(rec, ids, policy, S, b)
+    assert np.array_equal(hi, ehi), np.nonzero(hi != ehi)[0][:5]
+    assert np.array_equal(lo, elo), np.nonzero(lo != elo)[0][:5]
+
+
 def test_window_setter_errors():
     from paper_2405_03605_gb300 import ga
     s = gpu_run(RunShape(rows=2, cols=2))
