@@ -96,13 +96,24 @@ __device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, u
     return make_uint4(c0, c1, c2, c3);
 }
 
-__device__ __forceinline__ uint4 philox_rk(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
-                                           const RoundKeys &rk)
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
+
+__device__ __forceinline__ void mul_both(uint32_t a, uint32_t m, uint32_t &lo, uint32_t &hi)
+{
+    lo = a * m;
+    hi = __umulhi(a, m);
+}
+
+// Rounds r >= R0 of Philox on counter words c0..c3.
+template <int R0>
+__device__ __forceinline__ uint4 philox_rounds(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
+                                               const RoundKeys &rk)
 {
 #pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const uint32_t alo = c0 * 0xD2511F53u, ahi = __umulhi(c0, 0xD2511F53u);
-        const uint32_t blo = c2 * 0xCD9E8D57u, bhi = __umulhi(c2, 0xCD9E8D57u);
+    for (int r = R0; r < 10; ++r) {
+        uint32_t alo, ahi, blo, bhi;
+        mul_both(c0, kPhiloxM0, alo, ahi);
+        mul_both(c2, kPhiloxM1, blo, bhi);
         const uint32_t n0 = bhi ^ c1 ^ rk.k0[r];
         const uint32_t n2 = ahi ^ c3 ^ rk.k1[r];
         c1 = blo;
@@ -111,6 +122,12 @@ __device__ __forceinline__ uint4 philox_rk(uint32_t c0, uint32_t c1, uint32_t c2
         c2 = n2;
     }
     return make_uint4(c0, c1, c2, c3);
+}
+
+__device__ __forceinline__ uint4 philox_rk(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
+                                           const RoundKeys &rk)
+{
+    return philox_rounds<0>(c0, c1, c2, c3, rk);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -101,6 +101,58 @@ __device__ __forceinline__ void birth_draws(uint4 (&w)[Shape<N>::A], const RunPa
         w[ag] = philox_rk(g, island, (seg_lane + 32u * ag) | (kBirth << 16), p.run_id, rk);
 }
 
+// The same draws over many islands of one run and generation.  Counter (g, island, slot | purpose,
+// run): most of Philox's first three rounds does not see the island.  Round 1 multiplies g and
+// the slot word; round 2's second product has the factor hi(M0 g) ^ run ^ k1, and its first
+// output word, the factor of round 3's first product, is again made of the slot and g alone.
+// Those four of the twenty products (and two of the twenty XORs) are done once per warp and
+// generation; an island's draws take the other sixteen.  The lanes' words pass through an empty
+// asm: without it the compiler recomputes them in every unit rather than hold three registers
+// (island step of 16.8M agents: 98 us with them recomputed, 93 us held).
+template <int N>
+struct SlotDraws {
+    uint32_t h[Shape<N>::A];  // round 1: hi(M1 slot) ^ k0; XOR the island gives round 2's factor
+    uint32_t q[Shape<N>::A];  // round 3: hi of its first product, ^ k1
+    uint32_t l[Shape<N>::A];  //          and its low half
+    uint32_t v, w;            // the run's and generation's words of rounds 2 and 3
+};
+
+template <int N>
+__device__ __forceinline__ SlotDraws<N> slot_draws(const RunParams &p, const RoundKeys &rk, uint32_t g,
+                                                   uint32_t seg_lane)
+{
+    SlotDraws<N> s;
+    uint32_t alo, ahi, blo, bhi;
+    mul_both(g, kPhiloxM0, alo, ahi);
+    mul_both(ahi ^ p.run_id ^ rk.k1[0], kPhiloxM1, blo, bhi);
+    s.v = alo ^ rk.k1[1];
+    s.w = blo ^ rk.k0[2];
+#pragma unroll
+    for (int ag = 0; ag < Shape<N>::A; ++ag) {
+        uint32_t lo, hi;
+        mul_both((seg_lane + 32u * ag) | (kBirth << 16), kPhiloxM1, lo, hi);
+        s.h[ag] = hi ^ rk.k0[0];
+        mul_both(lo ^ bhi ^ rk.k0[1], kPhiloxM0, lo, hi);
+        s.q[ag] = hi ^ rk.k1[2];
+        s.l[ag] = lo;
+        asm volatile("" : "+r"(s.h[ag]), "+r"(s.q[ag]), "+r"(s.l[ag]));
+    }
+    return s;
+}
+
+template <int N>
+__device__ __forceinline__ void island_draws(uint4 (&w)[Shape<N>::A], const SlotDraws<N> &s,
+                                             const RoundKeys &rk, uint32_t island)
+{
+#pragma unroll
+    for (int ag = 0; ag < Shape<N>::A; ++ag) {
+        uint32_t alo, ahi, blo, bhi;
+        mul_both(s.h[ag] ^ island, kPhiloxM0, alo, ahi);
+        mul_both(ahi ^ s.v, kPhiloxM1, blo, bhi);
+        w[ag] = philox_rounds<3>(bhi ^ s.w, blo, s.q[ag] ^ alo, s.l[ag], rk);
+    }
+}
+
 // Evaluation, tournament, copy, mutation and hstrat deposit of one generation, in place.
 // Closed-form curation site, called only for agents whose counter differs from the
 // generation (never in synchronous runs); kept out of line so the common path stays a load.
@@ -133,6 +185,7 @@ __device__ __forceinline__ void reproduce(uint32_t (&rec)[Shape<N>::A][2 + SW],
 #pragma unroll
     for (int ag = 0; ag < A; ++ag) trait[ag] = static_cast<int>(rec[ag][0]);
     uint32_t win[A];
+    int won[A];  // the winner's trait
 #pragma unroll
     for (int ag = 0; ag < A; ++ag) {
         uint32_t best = 0;
@@ -183,6 +236,7 @@ __device__ __forceinline__ void reproduce(uint32_t (&rec)[Shape<N>::A][2 + SW],
             }
         }
         win[ag] = best;
+        won[ag] = best_trait;
     }
 
     // copy the winner's record
@@ -191,6 +245,17 @@ __device__ __forceinline__ void reproduce(uint32_t (&rec)[Shape<N>::A][2 + SW],
     for (int ag = 0; ag < A; ++ag) {
 #pragma unroll
         for (int k = 0; k < LW; ++k) {
+            // the winner's trait came with the tournament (but where a float run of run-time
+            // size loaded a NaN, no draw may have set it), and with uniform counters its
+            // counter is g
+            if (k == 0 && !(TS == 0 && MODEL == 1)) {
+                child[ag][0] = static_cast<uint32_t>(won[ag]);
+                continue;
+            }
+            if (k == 1 && CF == 0) {
+                child[ag][1] = g;
+                continue;
+            }
             if constexpr (N <= 32) {
                 child[ag][k] = __shfl_sync(mask, rec[0][k], static_cast<int>(win[ag]), SEG);
             } else {
@@ -549,6 +614,7 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
     __syncthreads();
 
     const uint2 dmask = gen_mask_at(p, 0u);
+    const SlotDraws<N> sd = slot_draws<N>(p, rk, p.g0, seg_lane);
     // UNROLL: fully unrolled over the block's units, so the double-buffer index, the
     // shared-memory offsets of each unit and the loop control become constants (94.2 against
     // 101.7 us per generation of 16.8M agents with the loop kept rolled; 3-10% on the other
@@ -575,7 +641,7 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
             if (!valid) break;  // only lanes of a missing last island; later units are past too
         }
         uint4 w[A];
-        birth_draws<N>(w, p, rk, p.g0, island, seg_lane);
+        island_draws<N>(w, sd, rk, island);
         cp_async_wait<1>();  // this unit's records have landed
         uint32_t rec[A][LW];
 #pragma unroll
