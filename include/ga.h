@@ -167,20 +167,24 @@ int ga_async_window(ga_run *run, uint32_t window);
 
 /*
  * Resident stepping (Sec. 2: each processor keeps its population in place and exchanges only
- * migrants with its neighbours).  A synchronous run whose islands all fit on the GPU at once
- * can step a whole chunk of up to 4,096 generations in one cooperative launch: every island
- * stays in registers, and on each migration generation an island pushes the member each
- * neighbour draws into that neighbour's mailbox (one 16-byte atomic write) and reads its own
- * four mailboxes, waiting until each holds the record of the current generation.  Results are
- * bit-identical to the streamed launches.  Eligible: GA_SYNC, 16-byte records, island sizes
- * 8 to 64, counters equal to the generation, at most 8,192 islands, and a grid that the
- * device can hold resident; the mailboxes (128 bytes per island) are part of the workspace of
- * such runs.
- *   GA_RESIDENT_AUTO  (default) resident launches whenever eligible;
+ * migrants with its neighbours).  A synchronous run whose islands all fit in the GPU's shared
+ * memory can step a whole chunk of up to 4,096 generations in one cooperative launch: every
+ * island stays on its SM, and on each migration generation an island pushes the member each
+ * neighbour draws into that neighbour's mailbox and reads its own four mailboxes, waiting until
+ * each holds the record of the current generation.  Results are bit-identical to the streamed
+ * launches.
+ *   GA_RESIDENT_AUTO  (default) resident launches where they are faster: GA_SYNC, counters equal
+ *                     to the generation, island sizes 8 to 64, a population that the device
+ *                     holds at once, and an interval between migrations short enough for its
+ *                     size (with migration every generation up to 65,536 islands)
  *   GA_RESIDENT_OFF   one launch per migration interval, the population streamed;
  *   GA_RESIDENT_ON    resident launches; ga_step returns GA_EUNSUPPORTED if not eligible.
+ * Eligible for GA_RESIDENT_ON: GA_SYNC, 16-byte records, island sizes 8 to 64, counters equal to
+ * the generation, at most 8,192 islands, of which at most 40 of 32 agents and 32 of 64 agents
+ * for each SM of the device; the mailboxes (128 bytes per island) are part of the workspace of
+ * such runs.  Other runs keep theirs in the population buffer that the launch writes at its end.
  * wait_limit_us bounds every wait for a mailbox (wall clock, default 1,000,000 = 1 s): when
- * it runs out the launch records GA_ETIMEOUT, every block leaves at its next migration
+ * it runs out the launch records GA_ETIMEOUT, every warp leaves at its next migration
  * generation, the population is undefined, and the next ga_sync returns GA_ETIMEOUT (the
  * run can then be reset or loaded and stepped again).  Errors: GA_EINVAL (mode, limit 0).
  */
@@ -191,9 +195,9 @@ int ga_resident_policy(ga_run *run, uint32_t mode, uint32_t wait_limit_us);
 
 /*
  * Fault injection for testing the bounded waits above (the paper has no counterpart): in
- * resident launches, island `island` never pushes its emigrants, so its four neighbours wait
- * for mailboxes that nothing fills until their limit runs out.  0xFFFFFFFF (the default)
- * turns it off.  Errors: GA_EINVAL (island out of range).
+ * resident launches of runs that GA_RESIDENT_ON accepts (others stream while it is set), island
+ * `island` never pushes its emigrants, so its four neighbours wait for mailboxes that nothing
+ * fills until their limit runs out.  0xFFFFFFFF (the default) turns it off.  Errors: GA_EINVAL (island out of range).
  */
 int ga_inject_lost_migrants(ga_run *run, uint32_t island);
 

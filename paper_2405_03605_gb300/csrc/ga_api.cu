@@ -142,32 +142,37 @@ cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t stream)
     return cudaMallocFromPoolAsync(p, bytes, pool, stream);
 }
 
-int step_run(ga_run *run, uint32_t n_gens, cudaStream_t stream)
+int step_run(ga_run *run, uint32_t n_gens, cudaStream_t stream, bool shared)
 {
     if (run->cfg.mode != GA_SYNC) return async_step(run, n_gens, stream);
     if (run->generation + n_gens > 0xFFFFFFFFull) return GA_EINVAL;
     // resident launches: one cooperative launch per chunk of the site table
     bool resident = false;
+    ResidentPlan plan = {};
     if (n_gens > 0 && run->resident_mode != GA_RESIDENT_OFF) {
-        const bool wanted = run->resident_mode == GA_RESIDENT_ON || run->n_islands <= kResidentAutoIslands;
-        resident = wanted && resident_possible(run, nullptr);
+        const bool eligible = resident_eligible(run), dropping = run->drop_island != 0xFFFFFFFFu;
+        bool wanted = eligible;
+        if (run->resident_mode == GA_RESIDENT_AUTO && !(eligible && dropping))
+            wanted = (eligible || (!shared && !dropping && n_gens >= kResidentAutoGens)) && resident_pays(run);
+        resident = wanted && resident_plan(run, plan);
         if (run->resident_mode == GA_RESIDENT_ON && !resident) return GA_EUNSUPPORTED;
     }
     while (n_gens > 0) {
-        // curation sites of the next chunk of generations, computed on the device once
         const uint32_t chunk = n_gens < kSiteTableCap ? n_gens : kSiteTableCap;
-        int rc = cuda_rc(launch_site_table(run, static_cast<uint32_t>(run->generation), chunk, stream));
-        if (rc != GA_OK) return rc;
-        run->sites_base = run->generation;
         if (resident) {
-            rc = cuda_rc(launch_resident(run, run->pop[run->cur], run->pop[run->cur ^ 1],
-                                         static_cast<uint32_t>(run->generation), chunk, stream));
+            run->sites_base = run->generation;
+            const int rc = cuda_rc(launch_resident(run, plan, run->pop[run->cur], run->pop[run->cur ^ 1],
+                                                   static_cast<uint32_t>(run->generation), chunk, stream));
             if (rc != GA_OK) return rc;
             run->cur ^= 1;
             run->generation += chunk;
             n_gens -= chunk;
             continue;
         }
+        // curation sites of the next chunk of generations, computed on the device once
+        int rc = cuda_rc(launch_site_table(run, static_cast<uint32_t>(run->generation), chunk, stream));
+        if (rc != GA_OK) return rc;
+        run->sites_base = run->generation;
         uint32_t left = chunk;
         while (left > 0) {
             const uint64_t g = run->generation;
@@ -282,6 +287,7 @@ int ga_create(const ga_config *cfg, void *workspace, size_t workspace_bytes, ga_
     run->d_flag = reinterpret_cast<int *>(base + ga::kStatusBytes / 2);
     run->d_sites = reinterpret_cast<int32_t *>(base + ga::kStatusBytes);
     run->d_masks = reinterpret_cast<uint2 *>(base + ga::kMaskOffset);
+    run->d_abort = reinterpret_cast<uint32_t *>(base + ga::kStatusBytes / 4);
     run->resident_state = nullptr;
     if (cfg->mode == GA_SYNC &&
         ga::resident_state_bytes(run->n_islands, run->record_bytes) != 0)

@@ -671,7 +671,7 @@ int ga_batch_step(ga_batch *b, uint32_t n_gens)
         size_t k = b->classes.size();
         for (ga_run *r : b->runs) {
             if (!ga::solo(r)) continue;
-            const int rs = ga::step_run(r, n_gens, b->side[k++ % b->side.size()]);
+            const int rs = ga::step_run(r, n_gens, b->side[k++ % b->side.size()], true);
             if (rs != GA_OK) return rs;
         }
     }

@@ -243,6 +243,20 @@ __device__ __forceinline__ int curation_site(uint32_t policy, uint32_t s, uint32
     return static_cast<int>(S >> 1) + tilted_site(S >> 1, T >> 1);
 }
 
+// Site-table entry of rank T: its curation site and, where `mask` is given (sites * bits <= 64),
+// the bits of surface words 0 and 1 that its deposit overwrites.
+__device__ __forceinline__ void store_curation_site(uint32_t policy, uint32_t s, uint32_t S, uint32_t T,
+                                                    uint32_t bits, int32_t *site_out, uint2 *mask)
+{
+    const int site = curation_site(policy, s, S, T);
+    *site_out = site;
+    if (mask) {
+        const uint32_t pos = site >= 0 ? static_cast<uint32_t>(site) * bits : 0u;
+        const uint32_t m = site >= 0 ? ((1u << bits) - 1u) << (pos & 31u) : 0u;
+        *mask = make_uint2(pos < 32u ? m : 0u, pos < 32u ? 0u : m);
+    }
+}
+
 // Unsigned division by the torus width as a multiply and shifts, with the magic number of
 // Granlund and Montgomery ("Division by invariant integers using multiplication", PLDI
 // 1994, the round-up method for a 32-bit divisor d >= 2): l = ceil(log2 d),

@@ -36,8 +36,9 @@ struct ga_run {
     bool counters_uniform;  // every agent's counter equals `generation` (founder, sync steps)
     int *d_flag;         // device scratch word for ga_load's counter check (workspace header)
     uint2 *d_masks;      // deposit masks of generation sites_base + i (workspace header)
-    // resident stepping (ga_resident.cu): abort word and mailboxes (null when the run is too
-    // large or not synchronous), policy, wait limit and the fault-injection island
+    // resident stepping (ga_resident.cu): abort word (workspace header), mailboxes (null when
+    // the run is too large or not synchronous), policy, wait limit and the fault-injection island
+    uint32_t *d_abort;
     void *resident_state;
     uint32_t resident_mode;
     uint32_t resident_wait_us;
@@ -97,8 +98,10 @@ cudaError_t launch_island_step(ga_run *run, const void *src, void *dst, uint32_t
 // Fill the site table with the curation sites of generations [g0, g0 + count).
 cudaError_t launch_site_table(ga_run *run, uint32_t g0, uint32_t count, cudaStream_t stream);
 // Advance one run by n_gens generations with the single-run kernels on `stream` (the body of
-// ga_step; the batch uses it for members that fill the GPU on their own).
-int step_run(ga_run *run, uint32_t n_gens, cudaStream_t stream);
+// ga_step; the batch uses it for members that fill the GPU on their own).  shared: other launches
+// step beside these ones, so a resident launch may not take the whole GPU (only the runs that
+// GA_RESIDENT_ON accepts step resident).
+int step_run(ga_run *run, uint32_t n_gens, cudaStream_t stream, bool shared = false);
 cudaError_t launch_mrca(ga_run *run, const uint32_t *d_ids, uint32_t n, uint32_t *d_lo,
                         uint32_t *d_hi, void *scratch);
 size_t mrca_scratch_bytes(const ga_run *run, uint32_t n);
@@ -113,18 +116,30 @@ cudaError_t launch_island_async(ga_run *run, const void *src, void *dst, uint32_
                                 cudaStream_t stream);
 int async_step(ga_run *run, uint32_t n_gens, cudaStream_t stream);
 
-// Resident stepping (ga_resident.cu).  Runs of at most kResidentMaxIslands islands with
-// 16-byte records get the mailbox state in their workspace; GA_RESIDENT_AUTO uses resident
-// launches up to kResidentAutoIslands islands.
+// Resident stepping (ga_resident.cu).  Runs of at most kResidentMaxIslands islands with 16-byte
+// records have mailboxes in their workspace.
 constexpr uint32_t kResidentMaxIslands = 8192;
-constexpr uint32_t kResidentAutoIslands = 8192;
+// GA_RESIDENT_AUTO streams calls of fewer generations for runs without them: the launches around
+// a resident chunk cost as much as a few streamed generations (9,991 islands of 32, calls of 1,
+// 2, 4 and 8 generations: 17, 25, 35 and 61 us streamed, 22, 25, 29 and 41 us resident).
+constexpr uint32_t kResidentAutoGens = 4;
 size_t resident_state_bytes(uint32_t n_islands, uint32_t record_bytes);
-// The run can step resident now: state present, synchronous, counters equal to the generation,
-// a kernel for its island size, and its grid co-resident on the device.
-bool resident_possible(const ga_run *run, uint32_t *blocks);
-// Generations [g0, g0 + n_gens) of the whole run in one cooperative launch (src -> dst).
-cudaError_t launch_resident(ga_run *run, const void *src, void *dst, uint32_t g0, uint32_t n_gens,
-                            cudaStream_t stream);
+struct ResidentPlan {
+    uint32_t units, blocks;
+    size_t shared_bytes;
+};
+// What GA_RESIDENT_ON accepts and GA_RESIDENT_AUTO steps resident at any length: a synchronous run
+// with mailboxes in its workspace, counters equal to the generation, islands of 8 to 64 agents
+// and at most as many islands per SM as that mode has always taken.
+bool resident_eligible(const ga_run *run);
+// Whether GA_RESIDENT_AUTO prefers resident launches: by migration interval and population.
+bool resident_pays(const ga_run *run);
+// A launch shape that holds the whole run on the device at once, if there is one.
+bool resident_plan(const ga_run *run, ResidentPlan &plan);
+// Generations [g0, g0 + n_gens) of the whole run in one cooperative launch (src -> dst), after
+// filling their site table.
+cudaError_t launch_resident(ga_run *run, const ResidentPlan &plan, const void *src, void *dst, uint32_t g0,
+                            uint32_t n_gens, cudaStream_t stream);
 
 // Curation sites of ranks [t0, t0 + count); with d_masks (S * bits <= 64) also the deposit
 // masks of those ranks.

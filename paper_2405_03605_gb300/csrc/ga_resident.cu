@@ -1,43 +1,50 @@
-// ga_resident.cu -- resident stepping: a run whose islands all fit on the GPU at once stays
-// in registers for a whole chunk of generations, in one cooperative launch, and its islands
-// trade migrants through mailboxes in global memory (L2) instead of through launch
-// boundaries.  The paper's processors keep their populations in place and exchange only
-// migrants with their neighbours (Sec. 2); this is that arrangement on the GPU, for runs
-// small enough that a launch per generation would be bound by launch latency.
+// ga_resident.cu -- resident stepping: a run whose population fits in the SMs' shared memory
+// stays there for a whole chunk of generations, in one cooperative launch, and its islands
+// trade migrants through mailboxes in global memory (L2) instead of through launch boundaries.
+// The paper's processors keep their populations in place and exchange only migrants with their
+// neighbours (Sec. 2); this is that arrangement on the GPU.  A launch per generation cannot
+// follow it there: launches on one stream start at least 4 us apart, and a run of 320,000
+// agents needs 2 us of arithmetic per generation.
 //
-// Scope: synchronous runs whose counters all equal the generation, 16-byte records (trait or
-// float fitness, counter, 64-bit surface).  Results are bit-identical to the streamed
-// kernels: the same draws, landing slots, tournaments, mutations and deposits.
+// Scope: synchronous runs whose counters all equal the generation, any record size, islands of
+// 8 to 64 agents.  Results are bit-identical to the streamed kernels: the same draws, landing
+// slots, tournaments, mutations and deposits.
 //
-// Islands of 32 and 64 agents take resident_warp_kernel: one island per warp, which pushes,
-// polls and lands its own migrants with no block barrier (described at the kernel).
-// Islands of 8 and 16 agents share warps and take resident_kernel.  Its block: WARPS island
-// warps (the mapping of step_block) plus BK bookkeeping warps, one lane per (island,
-// direction).  On each migration generation g:
-//   A. block barrier: the bookkeeping lanes have prepared g's sends (below) and the island
-//      warps hold the state before g;
-//   B. island warps push: for each direction d the member that the neighbour R = nb(I, d)
-//      draws (bits 8..15 of word 3 of R's slot-(d^1) birth draw) is written, with one 128-bit
-//      atomic exchange, into R's mailbox for direction d^1 and generation parity (g/k) & 1;
-//      bookkeeping lanes poll their island's mailbox for direction d (128-bit atomic reads)
-//      until it holds a record whose counter is g -- the record is its own ready flag, as
-//      every counter equals the generation -- and place it at the landing slot (the partial
-//      Fisher-Yates draw of the synchronous mode);
-//      meanwhile the island warps compute g's birth draws, which need nothing exchanged;
-//   C. block barrier; island warps land the immigrants and reproduce g and the generations up
-//      to the next migration, while the bookkeeping lanes prepare the next migration
-//      generation's sends (two Philox calls per lane: the neighbour's draw for the emigrant
-//      and the island's own for the landing slot).
-// Every island pushes before it polls, and a cooperative launch keeps every block resident,
-// so each poll is answered once the neighbour reaches the same generation.  Mailboxes are
-// double-buffered by generation parity: a sender can only overwrite a parity slot after it
-// has received the receiver's next push, which the receiver makes after reading that slot.
+// Mapping: each warp holds a few consecutive islands (units of Shape<N>::P) in shared memory
+// for the whole launch and works through them one unit at a time, as step_units does.  The
+// migration bookkeeping is done for all the warp's islands at once, one (island, direction)
+// pair per lane.  On a migration generation g the warp
+//   1. pushes: lane (I, d) writes the member that the neighbour in direction d draws into that
+//      neighbour's mailbox for direction d ^ 1 and this migration's parity;
+//   2. draws what needs no arrival: the next migration's emigrants and landing slots (they
+//      depend on no state) and its first islands' births;
+//   3. polls: lane (I, d) reads I's mailbox for direction d until it holds generation g;
+//   4. lands the arrivals in its islands' records (shared memory) and reproduces.
+// Warps never wait for one another inside a block, and there is no block barrier.
+//
+// Mailboxes: a 16-byte record is its own ready flag (its counter is g); wider records travel as
+// three 16-byte chunks of three words and the generation, their counter being g.  Each chunk is
+// one 128-bit relaxed store and load at GPU scope, so it is seen whole or not at all.  They are
+// double-buffered by migration parity: a sender can only overwrite a chunk after it has received
+// the receiver's next push, which the receiver makes after reading that chunk.  Every island
+// pushes before it polls and the cooperative launch keeps every warp resident, so each poll is
+// answered once the neighbour reaches the same generation.  Runs without mailboxes in their
+// workspace (wider records, more than 8,192 islands) keep them in the destination buffer,
+// each island's in the place of its own records: those are written when the launch ends, by
+// the warp that has read the island's last arrival.
 //
 // Waits are bounded: a poll gives up after the run's wait limit (wall clock, %globaltimer),
 // records GA_ETIMEOUT in the status word and sets the launch's abort word; every poll also
-// watches the abort word, so once one block gives up every block leaves at its next
-// migration generation.  The population is then undefined; the status is returned by the
-// next ga_sync.
+// watches the abort word, so once one warp gives up every warp leaves at its next migration
+// generation.  The population is then undefined; the status is returned by the next ga_sync.
+//
+// What bounds it: small runs the two L2 trips of a migration (32x32 torus of 32-agent islands:
+// 1.23 us per generation), larger ones issue (9,991 islands of 32: 192 warp-instructions per
+// island and generation at 56% issue, 2.8 us per generation, 7.2 us with one launch each).
+// Per generation, launches before and now: 262,000 agents 6.2 and 2.7 us, 600,000 6.5 and 4.8,
+// 1,000,000 10.3 and 7.4; 48-byte records 33,000 4.2 and 1.6, 262,000 8.3 and 3.2, 600,000
+// 12.8 and 6.2.  48 or 40 registers instead of 64 (more warps, fewer islands each) are slower
+// throughout: 718 and 734 us against 710 us for 250 generations of 9,991 islands.
 #include "ga_device.cuh"
 #include "ga_internal.h"
 #include "ga_island.cuh"
@@ -49,14 +56,18 @@ RunParams run_params(const ga_run *run, const void *src, void *dst, uint32_t g0,
 
 namespace {
 
+constexpr uint32_t kWarps = 4;  // per block
+
 struct ResidentArgs {
     RunParams r;
     RoundKeys rk;
-    uint4 *mail;             // [2][n_islands * 4] mailboxes (all ones when empty)
-    uint32_t *abort_word;    // 0; set to 1 by a block that gave up waiting
+    uint4 *mail;             // mailboxes: island i's from mail + i * mail_stride
+    uint32_t mail_stride;    // [parity][direction][chunk] of an island, in 16-byte chunks
+    uint32_t *abort_word;    // 0; set to 1 by a warp that gave up waiting
     unsigned long long wait_ns;
     uint32_t every_k, per_neighbor;
     uint32_t drop_island;    // fault injection: this island's pushes are dropped (~0u: none)
+    uint32_t units;          // units of Shape<N>::P islands per warp
 };
 
 __device__ __forceinline__ unsigned long long global_ns()
@@ -66,50 +77,35 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
-// 128-bit atomic read: a compare-and-swap of all ones with all ones never changes memory
-// (a record is all ones only when its mailbox is empty) and returns the 16 bytes at once.
-__device__ __forceinline__ uint4 read128(uint4 *p)
+// 128-bit relaxed accesses at GPU scope, each one memory operation: the reader sees all of a
+// 16-byte chunk or none of it.
+__device__ __forceinline__ uint4 load128(const uint4 *p)
 {
     unsigned long long lo, hi;
-    const unsigned long long ones = ~0ull;
-    asm volatile("{\n\t.reg .b128 cv, ov;\n\t"
-                 "mov.b128 cv, {%2, %3};\n\t"
-                 "atom.relaxed.gpu.global.cas.b128 ov, [%4], cv, cv;\n\t"
-                 "mov.b128 {%0, %1}, ov;\n\t}"
-                 : "=l"(lo), "=l"(hi) : "l"(ones), "l"(ones), "l"(p) : "memory");
+    asm volatile("{\n\t.reg .b128 v;\n\t"
+                 "ld.relaxed.gpu.global.b128 v, [%2];\n\t"
+                 "mov.b128 {%0, %1}, v;\n\t}"
+                 : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
     return make_uint4(static_cast<uint32_t>(lo), static_cast<uint32_t>(lo >> 32),
                       static_cast<uint32_t>(hi), static_cast<uint32_t>(hi >> 32));
 }
 
-// 128-bit atomic write (exchange; the old contents are not needed).
-__device__ __forceinline__ void write128(uint4 *p, uint4 v)
+__device__ __forceinline__ void store128(uint4 *p, uint4 v)
 {
-    [[maybe_unused]] unsigned long long lo, hi;
-    const unsigned long long vlo = static_cast<unsigned long long>(v.x) |
-                                   (static_cast<unsigned long long>(v.y) << 32);
-    const unsigned long long vhi = static_cast<unsigned long long>(v.z) |
-                                   (static_cast<unsigned long long>(v.w) << 32);
-    asm volatile("{\n\t.reg .b128 nv, ov;\n\t"
-                 "mov.b128 nv, {%2, %3};\n\t"
-                 "atom.relaxed.gpu.global.exch.b128 ov, [%4], nv;\n\t"
-                 "mov.b128 {%0, %1}, ov;\n\t}"
-                 : "=l"(lo), "=l"(hi) : "l"(vlo), "l"(vhi), "l"(p) : "memory");
+    const unsigned long long lo = static_cast<unsigned long long>(v.x) | (static_cast<unsigned long long>(v.y) << 32);
+    const unsigned long long hi = static_cast<unsigned long long>(v.z) | (static_cast<unsigned long long>(v.w) << 32);
+    asm volatile("{\n\t.reg .b128 v;\n\t"
+                 "mov.b128 v, {%0, %1};\n\t"
+                 "st.relaxed.gpu.global.b128 [%2], v;\n\t}"
+                 :: "l"(lo), "l"(hi), "l"(p) : "memory");
 }
 
-__device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t *p)
+__device__ __forceinline__ uint32_t load_relaxed(const uint32_t *p)
 {
     uint32_t v;
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-
-template <int N, int WARPS>
-struct ResidentShape {
-    static constexpr int BI = WARPS * Shape<N>::P;  // islands per block
-    static constexpr int ML = 4 * BI;               // bookkeeping lanes
-    static constexpr int BK = (ML + 31) / 32;       // bookkeeping warps
-    static constexpr int THREADS = (WARPS + BK) * 32;
-};
 
 // Next migration generation at or after g (~0u: none before `end`).
 __device__ __forceinline__ uint32_t next_migration(uint32_t g, uint32_t end, uint32_t k, uint32_t on)
@@ -120,64 +116,77 @@ __device__ __forceinline__ uint32_t next_migration(uint32_t g, uint32_t end, uin
     return m < end ? static_cast<uint32_t>(m) : ~0u;
 }
 
-template <int N, int TS, int MODEL, int WARPS>
-__global__ void __launch_bounds__(ResidentShape<N, WARPS>::THREADS)
-resident_kernel(const ResidentArgs a)
-{
-    using RS = ResidentShape<N, WARPS>;
-    constexpr int A = Shape<N>::A, P = Shape<N>::P, SEG = Shape<N>::SEG;
-    constexpr int BI = RS::BI, ML = RS::ML, LW = 4;
-    static_assert(N <= 16, "islands of 32 and 64 agents take resident_warp_kernel");
-    __shared__ uint32_t s_send_e[ML];    // member of the island that neighbour R draws
-    __shared__ uint32_t s_send_box[ML];  // R's mailbox index: R * 4 + (d ^ 1)
-    __shared__ uint4 s_in[BI * N];       // arrivals by (island, slot)
-    __shared__ uint32_t s_hit[BI];       // slots that received one, by island
-    __shared__ int s_abort;
-    const RunParams &p = a.r;
+template <int SW>
+struct Record {
+    static constexpr int LW = 2 + SW;
+    static constexpr int Q = (LW + 3) / 4;       // 128-bit words of a record
+    static constexpr int C = Q == 1 ? 1 : 3;     // 128-bit chunks of a mailbox
+};
 
+// Shared memory of one warp, in bytes: its records, then by (island, direction) the neighbour,
+// the landing slots of two migrations and the emigrant.
+template <int N, int SW>
+__host__ __device__ constexpr uint32_t warp_bytes(uint32_t islands)
+{
+    return islands * (N * Record<SW>::Q * 16u + 4u * (4u + 2u + 1u) + 4u);
+}
+
+template <int N, int SW, int TS, int MODEL>
+__global__ void __launch_bounds__(kWarps * 32, 8) resident_kernel(const ResidentArgs a)
+{
+    constexpr int A = Shape<N>::A, P = Shape<N>::P, SEG = Shape<N>::SEG;
+    constexpr int LW = Record<SW>::LW, Q = Record<SW>::Q, C = Record<SW>::C;
+    extern __shared__ uint4 s_all[];
+    const RunParams &p = a.r;
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
-    const bool island_warp = warp < static_cast<uint32_t>(WARPS);
-    const uint32_t island0 = blockIdx.x * BI;
+    const uint32_t seg_lane = lane % SEG;
+    const uint32_t per_warp = a.units * P;
+    const uint32_t first = (blockIdx.x * kWarps + warp) * per_warp;
+    if (first >= p.n_islands) return;  // whole warps
+    const uint32_t count = min(per_warp, p.n_islands - first);
+    const uint32_t pairs = count * 4u;  // (island, direction) pairs of the warp
     const uint32_t end = p.g0 + p.n_gens;
 
-    // island lanes
-    const uint32_t seg_lane = lane % SEG;
-    const uint32_t local = warp * P + lane / SEG;
-    const uint32_t island = island0 + local;
-    const bool valid = island_warp && island < p.n_islands;
-    const unsigned mask = __ballot_sync(0xffffffffu, valid);
+    uint8_t *mine = reinterpret_cast<uint8_t *>(s_all) + warp * warp_bytes<N, SW>(per_warp);
+    uint4 *recs = reinterpret_cast<uint4 *>(mine);
+    uint32_t *s_nb = reinterpret_cast<uint32_t *>(mine + per_warp * (N * Q * 16u));
+    uint8_t *s_slot = reinterpret_cast<uint8_t *>(s_nb + per_warp * 4u);  // [2][per_warp * 4]
+    uint8_t *s_e = s_slot + per_warp * 8u;
 
-    // bookkeeping lanes: (island t / 4, direction t % 4)
-    const uint32_t t = threadIdx.x - WARPS * 32u;
-    const bool bk = !island_warp && t < static_cast<uint32_t>(ML);
-    const unsigned bk_mask = __ballot_sync(0xffffffffu, bk);
-    const uint32_t md = t & 3u;
-    const uint32_t bk_isl = island0 + (t >> 2);
-    const bool bk_ok = bk && bk_isl < p.n_islands;
-    uint32_t bk_slot = 0;  // landing slot of this lane's direction at the prepared generation
+    for (uint32_t i = lane; i < count * (N * Q); i += 32u)
+        cp_async16(&recs[i], &p.src[static_cast<size_t>(first) * (N * Q) + i]);
+    cp_async_commit();
+    for (uint32_t idx = lane; idx < pairs; idx += 32u) {
+        const uint32_t isl = first + (idx >> 2), d = idx & 3u;
+        const uint32_t y = div_cols(isl, p.cols_m, p.cols_l), x = isl - y * p.cols;
+        const uint32_t yn = d == 0u ? (y == 0u ? p.rows - 1u : y - 1u)
+                          : d == 1u ? (y + 1u == p.rows ? 0u : y + 1u) : y;
+        const uint32_t xn = d == 2u ? (x + 1u == p.cols ? 0u : x + 1u)
+                          : d == 3u ? (x == 0u ? p.cols - 1u : x - 1u) : x;
+        const uint32_t nb = yn * p.cols + xn;
+        s_nb[idx] = in_bounds(nb < p.n_islands, p.status) ? nb : 0u;
+    }
+    __syncwarp();
 
-    // the bookkeeping lanes' share of migration generation gm: the emigrant the neighbour
-    // draws, where it goes, and this island's own landing slot for direction md
-    auto prepare = [&](uint32_t gm) {
-        uint32_t r = md;
-        if (bk_ok) {
-            const uint32_t y = div_cols(bk_isl, p.cols_m, p.cols_l), x = bk_isl - y * p.cols;
-            const uint32_t yn = md == 0u ? (y == 0u ? p.rows - 1u : y - 1u)
-                              : md == 1u ? (y + 1u == p.rows ? 0u : y + 1u) : y;
-            const uint32_t xn = md == 2u ? (x + 1u == p.cols ? 0u : x + 1u)
-                              : md == 3u ? (x == 0u ? p.cols - 1u : x - 1u) : x;
-            const uint32_t nb = yn * p.cols + xn;
-            const uint32_t un = philox_rk(gm, nb, (md ^ 1u) | (kBirth << 16), p.run_id, a.rk).w;
-            s_send_e[t] = (((un >> 8) & 0xFFu) * N) >> 8;
-            s_send_box[t] = nb * 4u + (md ^ 1u);
-            const uint32_t uo = philox_rk(gm, bk_isl, md | (kBirth << 16), p.run_id, a.rk).w;
-            r = md + (((uo >> 16) * static_cast<uint32_t>(N - md)) >> 16);
-        }
-        if (bk) {
+    // The draws of migration generation gm, two per (island, direction) pair and one per lane at
+    // a time: items [0, pairs) draw the member that the neighbour takes from this island (word 3,
+    // bits 8..15, of the neighbour's own draw for the slot facing it), items [pairs, 2 pairs) the
+    // landing slot of the arrival (the partial Fisher-Yates draw over [0, N) in direction order,
+    // among the island's four lanes).
+    auto prepare = [&](uint32_t gm, uint32_t par) {
+        for (uint32_t base = 0; base < 2u * pairs; base += 32u) {
+            const uint32_t item = base + lane;
+            const bool own = item >= pairs;
+            const uint32_t idx = own ? item - pairs : item;
+            const bool ok = item < 2u * pairs;
+            const uint32_t d = idx & 3u;
+            const uint32_t isl = own ? first + (idx >> 2) : s_nb[idx];
+            const uint32_t u = philox_rk(gm, isl, (own ? d : d ^ 1u) | (kBirth << 16), p.run_id, a.rk).w;
+            const uint32_t r = d + (((u >> 16) * static_cast<uint32_t>(N - d)) >> 16);
             uint32_t rr[4];
 #pragma unroll
-            for (int dd = 0; dd < 4; ++dd) rr[dd] = __shfl_sync(bk_mask, r, dd, 4);
-            uint32_t v[4];
+            for (int dd = 0; dd < 4; ++dd) rr[dd] = __shfl_sync(0xffffffffu, r, dd, 4);
+            uint32_t v[4], slot = 0;
 #pragma unroll
             for (int dd = 0; dd < 4; ++dd) {
                 uint32_t vd = dd, vr = rr[dd];
@@ -186,338 +195,254 @@ resident_kernel(const ResidentArgs a)
                     if (rr[e] == static_cast<uint32_t>(dd)) vd = v[e];
                     if (rr[e] == rr[dd]) vr = v[e];
                 }
-                if (static_cast<uint32_t>(dd) == md) bk_slot = vr;
+                if (static_cast<uint32_t>(dd) == d) slot = vr;
                 v[dd] = vd;
+            }
+            if (ok) {
+                if (own) s_slot[par * (per_warp * 4u) + idx] = static_cast<uint8_t>(slot);
+                else s_e[idx] = static_cast<uint8_t>((((u >> 8) & 0xFFu) * N) >> 8);
             }
         }
     };
+    // mailbox of island i for direction d, migration parity 0 (parity 1: 4 C chunks further)
+    auto box_of = [&](uint32_t i, uint32_t d) { return a.mail + static_cast<size_t>(i) * a.mail_stride + d * C; };
+    // this lane's first pair: its own mailbox and the neighbour's that it fills
+    uint4 *const box_in = box_of(first + (lane < pairs ? lane >> 2 : 0u), lane & 3u);
+    uint4 *const box_out = box_of(lane < pairs ? s_nb[lane] : first, (lane & 3u) ^ 1u);
 
-    uint32_t rec[A][LW];
-    if (valid) {
-#pragma unroll
-        for (int ag = 0; ag < A; ++ag) {
-            const uint4 v = __ldg(&p.src[static_cast<size_t>(island) * N + seg_lane + 32u * ag]);
-            rec[ag][0] = v.x;
-            rec[ag][1] = v.y;
-            rec[ag][2] = v.z;
-            rec[ag][3] = v.w;
-        }
-    }
-    if (threadIdx.x == 0) s_abort = 0;
     uint32_t gm = next_migration(p.g0, end, a.every_k, a.per_neighbor);
-    if (gm != ~0u) prepare(gm);
-
+    uint32_t par = 0;
+    if (gm != ~0u) prepare(gm, par);
+    cp_async_wait<0>();
+    __syncwarp();
     bool aborted = false;
     for (uint32_t it = 0; it < p.n_gens; ++it) {
         const uint32_t g = p.g0 + it;
+        uint2 dm = make_uint2(0u, 0u);
+        int site = -1;
+        if constexpr (SW == 2) dm = gen_mask_at(p, it);
+        else site = gen_site_at(p, it);
+        const SlotDraws<N> sd = slot_draws<N>(p, a.rk, g, seg_lane);
         uint4 w[A];
-        bool drawn = false;
-        if (g == gm) {  // the same generation for every thread of the block
-            __syncthreads();  // A
-            uint4 *box = a.mail + static_cast<size_t>((g / a.every_k) & 1u) * p.n_islands * 4u;
-            if (valid && island != a.drop_island) {
+        if (g == gm) {
+            __syncwarp();  // the islands' records, written by their own lanes, are pushed by others
+            for (uint32_t idx = lane; idx < pairs; idx += 32u) {
+                const uint4 *r = recs + ((idx >> 2) * N + s_e[idx]) * Q;
+                uint4 *box = (idx == lane ? box_out : box_of(s_nb[idx], (idx & 3u) ^ 1u)) + par * (4u * C);
+                if (first + (idx >> 2) != a.drop_island) {
+                    if constexpr (C == 1) {
+                        store128(box, r[0]);
+                    } else {
+                        const uint4 r0 = r[0], r1 = r[1];
+                        uint4 r2 = make_uint4(0u, 0u, 0u, 0u);
+                        if constexpr (Q == 3) r2 = r[2];
+                        store128(box, make_uint4(r0.x, r0.z, r0.w, g));
+                        store128(box + 1, make_uint4(r1.x, r1.y, r1.z, g));
+                        store128(box + 2, make_uint4(r1.w, r2.x, r2.y, g));
+                    }
+                }
+            }
+            const uint64_t after = static_cast<uint64_t>(g) + a.every_k;
+            const uint32_t gm_next = after < end ? static_cast<uint32_t>(after) : ~0u;
+            bool gave_up = false;
+            for (uint32_t base = 0; base < pairs; base += 32u) {
+                const uint32_t idx = base + lane;
+                const bool act = idx < pairs;
+                const uint4 *box = (base == 0u ? box_in : box_of(first + (act ? idx >> 2 : 0u), idx & 3u)) +
+                                   par * (4u * C);
+                uint4 in[C];
+                auto read = [&]() {
 #pragma unroll
-                for (int dd = 0; dd < 4; ++dd) {
-                    const uint32_t e = s_send_e[4u * local + dd];
-#pragma unroll
-                    for (int ag = 0; ag < A; ++ag) {
-                        if (seg_lane + 32u * ag == e) {
-                            const uint32_t dst = s_send_box[4u * local + dd];
-                            if (in_bounds(dst < p.n_islands * 4u, p.status))
-                                write128(box + dst, make_uint4(rec[ag][0], rec[ag][1], rec[ag][2], rec[ag][3]));
+                    for (int c = 0; c < C; ++c) in[c] = load128(box + c);
+                };
+                auto arrived = [&]() {
+                    if constexpr (C == 1) return in[0].y == g;
+                    else return in[0].w == g && in[1].w == g && in[2].w == g;
+                };
+                // while the pushes and the first reads travel: the next migration's draws and the
+                // first islands' birth draws.  An arrival is read right after the pushes, and a
+                // second time in between where the warp holds one unit and has nothing else to
+                // do (32x32 torus, 1,000 generations: 1,230 us, 1,255 with one early read,
+                // 1,292 with one read after the draws); wider records, three chunks each, are
+                // read once after the draws (256 sites, 5,893 islands: 651 us, 689 before them).
+                if (C == 1 && act) read();
+                if (base == 0u && gm_next != ~0u) prepare(gm_next, par ^ 1u);
+                uint4 again = make_uint4(0u, 0u, 0u, 0u);
+                if (C == 1 && act && a.units == 1u) again = load128(box);
+                if (C != 1 && act) read();
+                if (base == 0u) island_draws<N>(w, sd, a.rk, first + lane / SEG);
+                if (C == 1 && a.units == 1u && !arrived()) in[0] = again;
+                if (act && !arrived()) {
+                    const unsigned long long t0 = global_ns();
+                    for (uint32_t polls = 0;; ++polls) {
+                        read();
+                        const uint32_t ab = load_relaxed(a.abort_word);
+                        if (arrived()) break;
+                        if (ab != 0u) {
+                            gave_up = true;
+                            break;
+                        }
+                        if (global_ns() - t0 > a.wait_ns) {
+                            atomicCAS(p.status, 0, GA_ETIMEOUT);
+                            atomicExch(a.abort_word, 1u);
+                            gave_up = true;
+                            break;
+                        }
+                        if (polls >= 8u) __nanosleep(64);
+                    }
+                }
+                if (__any_sync(0xffffffffu, gave_up)) {
+                    aborted = true;
+                    break;
+                }
+                __syncwarp();  // every push has read its record
+                if (act) {
+                    const uint32_t slot = s_slot[par * (per_warp * 4u) + idx];
+                    uint4 *r = recs + ((idx >> 2) * N + slot) * Q;
+                    if (in_bounds(slot < static_cast<uint32_t>(N), p.status)) {
+                        if constexpr (C == 1) {
+                            r[0] = in[0];
+                        } else {
+                            r[0] = make_uint4(in[0].x, g, in[0].y, in[0].z);
+                            r[1] = make_uint4(in[1].x, in[1].y, in[1].z, in[2].x);
+                            if constexpr (Q == 3) r[2] = make_uint4(in[2].y, in[2].z, 0u, 0u);
                         }
                     }
                 }
             }
-            // the generation's birth draws need nothing from the neighbours: the island warps
-            // compute them while the bookkeeping lanes wait for the mailboxes
-            if (valid) {
-                birth_draws<N>(w, p, a.rk, g, island, seg_lane);
-                drawn = true;
-            }
-            uint4 imm = make_uint4(0u, 0u, 0u, 0u);
-            if (bk_ok) {
-                uint4 *mine = box + static_cast<size_t>(bk_isl) * 4u + md;
-                const unsigned long long t0 = global_ns();
-                for (uint32_t polls = 0;; ++polls) {
-                    // the abort word is read beside the mailbox, not after it: a poll that
-                    // finds nothing costs one round trip to L2, not two
-                    imm = read128(mine);
-                    const uint32_t ab = ld_relaxed_u32(a.abort_word);
-                    if (imm.y == g) break;
-                    if (ab != 0u) {
-                        s_abort = 1;
-                        break;
-                    }
-                    if (global_ns() - t0 > a.wait_ns) {
-                        atomicCAS(p.status, 0, GA_ETIMEOUT);
-                        atomicExch(a.abort_word, 1u);
-                        s_abort = 1;
-                        break;
-                    }
-                    if (polls >= 8u) __nanosleep(64);
-                }
-            }
-            if (bk) {
-                const uint32_t li = t >> 2;
-                uint32_t bit = 1u << bk_slot;
-                bit |= __shfl_xor_sync(bk_mask, bit, 1, 4);
-                bit |= __shfl_xor_sync(bk_mask, bit, 2, 4);
-                if (bk_ok && in_bounds(li * N + bk_slot < static_cast<uint32_t>(BI * N), p.status))
-                    s_in[li * N + bk_slot] = imm;
-                if (md == 0u) s_hit[li] = bit;
-            }
-            __syncthreads();  // C
-            if (s_abort) {
-                aborted = true;
-                break;
-            }
-            if (valid) {
-                const bool hit = ((s_hit[local] >> seg_lane) & 1u) != 0u;
-                const uint4 xq = s_in[local * N + seg_lane];
-                if (hit) {
-                    rec[0][0] = xq.x;
-                    rec[0][1] = xq.y;
-                    rec[0][2] = xq.z;
-                    rec[0][3] = xq.w;
-                }
-            }
-            gm = next_migration(g + 1u, end, a.every_k, a.per_neighbor);
-            if (gm != ~0u) prepare(gm);
-        }
-        if (valid) {
-            if (!drawn) birth_draws<N>(w, p, a.rk, g, island, seg_lane);
-            reproduce<N, 2, TS, MODEL, 0, 1>(rec, w, p, a.rk, island, seg_lane, mask, g, 0,
-                                             gen_mask_at(p, it));
-        }
-    }
-    if (valid && !aborted) {
-#pragma unroll
-        for (int ag = 0; ag < A; ++ag)
-            p.dst[static_cast<size_t>(island) * N + seg_lane + 32u * ag] =
-                make_uint4(rec[ag][0], rec[ag][1], rec[ag][2], rec[ag][3]);
-    }
-}
-
-// One island per warp (32 and 64 agents), no block barrier: on a migration generation g the
-// warp's lanes 0..3 compute, for direction d, the neighbour R = nb(I, d)'s own slot-(d^1)
-// birth draw (the member e_d it takes from I), and the lane holding member e_d pushes it into
-// R's mailbox for direction d^1 (one 128-bit atomic exchange); while those writes reach L2
-// the warp computes g's birth draws, the landing slots (the partial Fisher-Yates draw of the
-// synchronous mode, from the island's own slot-0..3 draws) and the next migration
-// generation's emigrant draws, none of which needs an arrival; lanes 0..3 read the island's
-// four mailboxes once right after the pushes (that read travels while the warp draws, so an
-// island whose neighbours got to g first has their records without a further round trip),
-// then poll until each holds the record of generation g, and every lane takes the arrival
-// meant for its slot by shuffles.  Warps never wait for one another inside a
-// block; each poll is bounded as in resident_kernel, and a warp that sees the abort word
-// leaves.
-template <int N, int TS, int MODEL, int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, 8)
-resident_warp_kernel(const ResidentArgs a)
-{
-    constexpr int A = Shape<N>::A, LW = 4;
-    static_assert(N >= 32, "one island per warp");
-    const RunParams &p = a.r;
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t island = blockIdx.x * WARPS + (threadIdx.x >> 5);
-    if (island >= p.n_islands) return;  // whole warps
-    const uint32_t end = p.g0 + p.n_gens;
-    const uint32_t d = lane & 3u;
-    const bool dir_lane = lane < 4u;
-
-    // torus neighbour of this island in direction d (lanes 0..3)
-    uint32_t nb = island;
-    if (dir_lane) {
-        const uint32_t y = div_cols(island, p.cols_m, p.cols_l), x = island - y * p.cols;
-        const uint32_t yn = d == 0u ? (y == 0u ? p.rows - 1u : y - 1u)
-                          : d == 1u ? (y + 1u == p.rows ? 0u : y + 1u) : y;
-        const uint32_t xn = d == 2u ? (x + 1u == p.cols ? 0u : x + 1u)
-                          : d == 3u ? (x == 0u ? p.cols - 1u : x - 1u) : x;
-        nb = yn * p.cols + xn;
-    }
-
-    uint32_t rec[A][LW];
-#pragma unroll
-    for (int ag = 0; ag < A; ++ag) {
-        const uint4 v = __ldg(&p.src[static_cast<size_t>(island) * N + lane + 32u * ag]);
-        rec[ag][0] = v.x;
-        rec[ag][1] = v.y;
-        rec[ag][2] = v.z;
-        rec[ag][3] = v.w;
-    }
-    // the member the neighbour in direction d draws from this island at migration generation
-    // gm (lanes 0..3; every lane computes it, so the draw is not a divergent branch and can
-    // overlap other work): it depends on no state, so it is drawn a migration ahead
-    auto emigrant = [&](uint32_t gm) {
-        const uint32_t un = philox_rk(gm, nb, (d ^ 1u) | (kBirth << 16), p.run_id, a.rk).w;
-        return (((un >> 8) & 0xFFu) * N) >> 8;
-    };
-    uint32_t nd[4];
-#pragma unroll
-    for (int dd = 0; dd < 4; ++dd) nd[dd] = __shfl_sync(0xffffffffu, nb, dd);
-    uint32_t gm = next_migration(p.g0, end, a.every_k, a.per_neighbor);
-    uint32_t e = emigrant(gm);
-    bool aborted = false;
-    for (uint32_t it = 0; it < p.n_gens; ++it) {
-        const uint32_t g = p.g0 + it;
-        const uint2 dm = gen_mask_at(p, it);  // the generation's deposit masks, read up front
-        uint4 w[A];
-        if (g == gm) {
-            uint4 *box = a.mail + static_cast<size_t>((g / a.every_k) & 1u) * p.n_islands * 4u;
-            // sends: lane holding the member e_d pushes it to the neighbour in direction d
-#pragma unroll
-            for (int dd = 0; dd < 4; ++dd) {
-                const uint32_t ed = __shfl_sync(0xffffffffu, e, dd);
-#pragma unroll
-                for (int ag = 0; ag < A; ++ag) {
-                    if (lane + 32u * ag == ed && island != a.drop_island &&
-                        in_bounds(nd[dd] < p.n_islands, p.status))
-                        write128(box + static_cast<size_t>(nd[dd]) * 4u + (static_cast<uint32_t>(dd) ^ 1u),
-                                 make_uint4(rec[ag][0], rec[ag][1], rec[ag][2], rec[ag][3]));
-                }
-            }
-            // an early read of the island's own mailboxes: an island that reaches g after its
-            // neighbours (the one that sets the pace) usually finds their records already there,
-            // and this read returns while the warp draws instead of after
-            uint4 *mine = box + static_cast<size_t>(island) * 4u + d;
-            uint4 early = make_uint4(0u, 0u, 0u, 0u);
-            if (dir_lane) early = read128(mine);
-            // while the neighbours' writes travel: the next migration's emigrant draws, this
-            // generation's birth draws and the landing slots, none of which needs an arrival
-            const uint32_t gm_next = next_migration(g + 1u, end, a.every_k, a.per_neighbor);
-            const uint32_t e_next = emigrant(gm_next);
-            birth_draws<N>(w, p, a.rk, g, island, lane);
-            // landing slots: partial Fisher-Yates over [0, N) in direction order from slot d's
-            // own draw (word 3 of lane d's first birth draw), the same on every lane
-            const uint32_t u = __shfl_sync(0xffffffffu, w[0].w, static_cast<int>(d));
-            const uint32_t r_own = d + (((u >> 16) * static_cast<uint32_t>(N - d)) >> 16);
-            uint32_t rr[4];
-#pragma unroll
-            for (int dd = 0; dd < 4; ++dd) rr[dd] = __shfl_sync(0xffffffffu, r_own, dd);
-            uint32_t v[4], slot[4];
-#pragma unroll
-            for (int dd = 0; dd < 4; ++dd) {
-                uint32_t vd = dd, vr = rr[dd];
-#pragma unroll
-                for (int e2 = 0; e2 < dd; ++e2) {
-                    if (rr[e2] == static_cast<uint32_t>(dd)) vd = v[e2];
-                    if (rr[e2] == rr[dd]) vr = v[e2];
-                }
-                slot[dd] = vr;
-                v[dd] = vd;
-            }
-            int from[A];
-#pragma unroll
-            for (int ag = 0; ag < A; ++ag) {
-                const uint32_t mine = lane + 32u * ag;
-                from[ag] = -1;
-#pragma unroll
-                for (int dd = 0; dd < 4; ++dd)
-                    if (slot[dd] == mine) from[ag] = dd;
-            }
-            // receives: lanes 0..3 wait for the records of generation g
-            uint4 imm = early;
-            bool gave_up = false;
-            if (dir_lane && imm.y != g) {
-                const unsigned long long t0 = global_ns();
-                for (uint32_t polls = 0;; ++polls) {
-                    imm = read128(mine);  // the abort word beside it, as in resident_kernel
-                    const uint32_t ab = ld_relaxed_u32(a.abort_word);
-                    if (imm.y == g) break;
-                    if (ab != 0u) {
-                        gave_up = true;
-                        break;
-                    }
-                    if (global_ns() - t0 > a.wait_ns) {
-                        atomicCAS(p.status, 0, GA_ETIMEOUT);
-                        atomicExch(a.abort_word, 1u);
-                        gave_up = true;
-                        break;
-                    }
-                    if (polls >= 8u) __nanosleep(64);
-                }
-            }
-            if (__any_sync(0xffffffffu, gave_up)) {
-                aborted = true;
-                break;
-            }
-            const uint32_t im[4] = {imm.x, imm.y, imm.z, imm.w};
-#pragma unroll
-            for (int ag = 0; ag < A; ++ag) {
-#pragma unroll
-                for (int k = 0; k < LW; ++k) {
-                    const uint32_t val = __shfl_sync(0xffffffffu, im[k], from[ag] < 0 ? 0 : from[ag]);
-                    if (from[ag] >= 0) rec[ag][k] = val;
-                }
-            }
+            if (aborted) break;
+            __syncwarp();
+            par ^= 1u;
             gm = gm_next;
-            e = e_next;
-        } else {
-            birth_draws<N>(w, p, a.rk, g, island, lane);
         }
-        reproduce<N, 2, TS, MODEL, 0, 1>(rec, w, p, a.rk, island, lane, 0xffffffffu, g, 0, dm);
-    }
-    if (!aborted) {
+        else island_draws<N>(w, sd, a.rk, first + lane / SEG);
+        uint4 *own = recs + lane * Q;
+        for (uint32_t u = 0; u < count; u += P, own += 32u * A * Q) {
+            const uint32_t li = u + lane / SEG;
+            unsigned mask = 0xffffffffu;
+            if constexpr (P > 1) {
+                mask = __ballot_sync(0xffffffffu, li < count);
+                if (li >= count) continue;  // lanes of a missing last island
+            }
+            const uint32_t island = first + li;
+            if (u != 0u) island_draws<N>(w, sd, a.rk, island);
+            uint32_t rec[A][LW];
 #pragma unroll
-        for (int ag = 0; ag < A; ++ag)
-            p.dst[static_cast<size_t>(island) * N + lane + 32u * ag] =
-                make_uint4(rec[ag][0], rec[ag][1], rec[ag][2], rec[ag][3]);
+            for (int ag = 0; ag < A; ++ag)
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    const uint4 v = own[32u * ag * Q + q];
+                    const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (4 * q + k < LW) rec[ag][4 * q + k] = w4[k];
+                }
+            // records wider than 16 bytes take the deposit in shared memory, below
+            if constexpr (SW == 2)
+                reproduce<N, SW, TS, MODEL, 0, 1>(rec, w, p, a.rk, island, seg_lane, mask, g, 0, dm);
+            else
+                reproduce<N, SW, TS, MODEL, 0, 0>(rec, w, p, a.rk, island, seg_lane, mask, g, -1);
+#pragma unroll
+            for (int ag = 0; ag < A; ++ag)
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    uint32_t w4[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) w4[k] = 4 * q + k < LW ? rec[ag][4 * q + k] : 0u;
+                    own[32u * ag * Q + q] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+                }
+            if constexpr (SW > 2) {
+                const uint32_t pos = static_cast<uint32_t>(site) * p.bits;
+                if (site >= 0 && in_bounds(pos + p.bits <= 32u * SW, p.status)) {
+                    const uint32_t m = p.dif_mask << (pos & 31u);
+#pragma unroll
+                    for (int ag = 0; ag < A; ++ag) {
+                        uint32_t *word = reinterpret_cast<uint32_t *>(own + 32u * ag * Q) + 2u + (pos >> 5);
+                        *word = (*word & ~m) | ((w[ag].w << (pos & 31u)) & m);
+                    }
+                }
+            }
+        }
     }
+    __syncwarp();
+    if (!aborted)
+        for (uint32_t i = lane; i < count * (N * Q); i += 32u)
+            p.dst[static_cast<size_t>(first) * (N * Q) + i] = recs[i];
 }
 
 using ResidentKernel = void (*)(ResidentArgs);
 
-template <int N, int WARPS>
-ResidentKernel pick_model(uint32_t model, uint32_t tsize)
+struct ResidentPick {
+    ResidentKernel k = nullptr;
+    uint32_t islands_per_unit = 1;
+    uint32_t bytes_per_island = 0;  // shared memory
+    uint32_t boxes = 0;             // 16-byte chunks of an island's mailboxes, both parities
+};
+
+template <int N, int SW>
+ResidentPick picked(ResidentKernel k)
 {
-    if (model == GA_MODEL_FITNESS) {  // the float-fitness model: islands of 16 to 64 agents
-        if constexpr (N >= 16)
-            return tsize == 5u ? resident_kernel<N, 5, 1, WARPS> : resident_kernel<N, 0, 1, WARPS>;
-        return nullptr;
-    }
-    return tsize == 5u ? resident_kernel<N, 5, 0, WARPS> : resident_kernel<N, 0, 0, WARPS>;
+    // the mailboxes fit in the place of the island's own records
+    static_assert(8 * Record<SW>::C <= N * Record<SW>::Q, "mailboxes larger than the island");
+    ResidentPick m;
+    m.k = k;
+    m.islands_per_unit = Shape<N>::P;
+    m.bytes_per_island = warp_bytes<N, SW>(1);
+    m.boxes = 8u * Record<SW>::C;
+    return m;
 }
 
-// Island warps per block: 4 (small grids spread over more SMs).
-constexpr int kResidentWarps = 4;
+// Tournament size 5 (the paper's) is compiled in; other sizes are read from the run.
+template <int N, int SW, int MODEL = 0>
+ResidentPick pick_ts(uint32_t tsize)
+{
+    return picked<N, SW>(tsize == 5u ? resident_kernel<N, SW, 5, MODEL> : resident_kernel<N, SW, 0, MODEL>);
+}
 
-// Islands of 32 and 64 agents: one island per warp, no bookkeeping warp and no block barrier
-// (2.10 against 2.49 us per generation for the block kernel on the 32x32 torus of 32-agent
-// islands); smaller islands share a warp and keep the block kernel.
+// The float-fitness model: 16-byte records, islands of 16 to 64 agents.  32-byte records: not
+// for islands of 8, whose mailboxes would not fit in the place of their records.
 template <int N>
-ResidentKernel pick_warp_model(uint32_t model, uint32_t tsize)
+ResidentPick pick_n(uint32_t surface_words, uint32_t model, uint32_t tsize)
 {
-    if (model == GA_MODEL_FITNESS)
-        return tsize == 5u ? resident_warp_kernel<N, 5, 1, kResidentWarps>
-                           : resident_warp_kernel<N, 0, 1, kResidentWarps>;
-    return tsize == 5u ? resident_warp_kernel<N, 5, 0, kResidentWarps>
-                       : resident_warp_kernel<N, 0, 0, kResidentWarps>;
+    if (model == GA_MODEL_FITNESS) {
+        if constexpr (N >= 16)
+            if (surface_words <= 2u) return pick_ts<N, 2, 1>(tsize);
+        return ResidentPick();
+    }
+    if (surface_words <= 2u) return pick_ts<N, 2>(tsize);
+    if (surface_words <= 6u) {
+        if constexpr (N >= 16) return pick_ts<N, 6>(tsize);
+        return ResidentPick();
+    }
+    return pick_ts<N, 8>(tsize);
 }
 
-ResidentKernel pick_resident(uint32_t island_size, uint32_t model, uint32_t tsize, uint32_t &threads,
-                             uint32_t &islands_per_block)
+ResidentPick pick(const ga_run *run)
 {
-    switch (island_size) {
-    case 8:
-        threads = ResidentShape<8, kResidentWarps>::THREADS;
-        islands_per_block = ResidentShape<8, kResidentWarps>::BI;
-        return pick_model<8, kResidentWarps>(model, tsize);
-    case 16:
-        threads = ResidentShape<16, kResidentWarps>::THREADS;
-        islands_per_block = ResidentShape<16, kResidentWarps>::BI;
-        return pick_model<16, kResidentWarps>(model, tsize);
-    case 32:
-        threads = kResidentWarps * 32;
-        islands_per_block = kResidentWarps;
-        return pick_warp_model<32>(model, tsize);
-    case 64:
-        threads = kResidentWarps * 32;
-        islands_per_block = kResidentWarps;
-        return pick_warp_model<64>(model, tsize);
-    default:
-        return nullptr;
+    const uint32_t sw = run->surface_words, model = run->cfg.model, ts = run->cfg.tournament_size;
+    switch (run->cfg.island_size) {
+    case 8: return pick_n<8>(sw, model, ts);
+    case 16: return pick_n<16>(sw, model, ts);
+    case 32: return pick_n<32>(sw, model, ts);
+    case 64: return pick_n<64>(sw, model, ts);
+    default: return ResidentPick();
     }
+}
+
+// Before a launch: the curation sites (and deposit masks) of its generations, every mailbox
+// empty (all ones) and the abort word clear.
+__global__ void resident_init_kernel(uint4 *__restrict__ mail, uint32_t n_islands, uint32_t stride,
+                                     uint32_t boxes, uint32_t *__restrict__ abort_word, uint32_t policy,
+                                     uint32_t log2_sites, uint32_t sites, uint32_t t0, uint32_t count,
+                                     int32_t *__restrict__ out, uint32_t bits, uint2 *__restrict__ masks)
+{
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, all = gridDim.x * blockDim.x;
+    if (t == 0u) *abort_word = 0u;
+    for (uint32_t i = t; i < count; i += all)
+        store_curation_site(policy, log2_sites, sites, t0 + i, bits, &out[i], masks ? &masks[i] : nullptr);
+    const uint32_t total = n_islands * boxes;
+    for (uint32_t i = t; i < total; i += all)
+        mail[static_cast<size_t>(i / boxes) * stride + i % boxes] = make_uint4(~0u, ~0u, ~0u, ~0u);
 }
 
 }  // namespace
@@ -525,57 +450,115 @@ ResidentKernel pick_resident(uint32_t island_size, uint32_t model, uint32_t tsiz
 size_t resident_state_bytes(uint32_t n_islands, uint32_t record_bytes)
 {
     if (record_bytes != 16u || n_islands > kResidentMaxIslands) return 0;
-    // abort word (256 bytes), then two parities of four 16-byte mailboxes per island
+    // 256 bytes, then two parities of four 16-byte mailboxes per island
     return 256u + static_cast<size_t>(n_islands) * 4u * 2u * 16u;
 }
 
-bool resident_possible(const ga_run *run, uint32_t *blocks_out)
+bool resident_eligible(const ga_run *run)
 {
     if (!run->resident_state || run->cfg.mode != GA_SYNC || !run->counters_uniform) return false;
-    uint32_t threads = 0, per_block = 0;
-    const ResidentKernel k =
-        pick_resident(run->cfg.island_size, run->cfg.model, run->cfg.tournament_size, threads, per_block);
-    if (!k) return false;
-    const uint32_t blocks = (run->n_islands + per_block - 1) / per_block;
-    int dev = 0, sms = 0, per_sm = 0;
+    const uint32_t N = run->cfg.island_size;
+    if (N < 8u || N > 64u) return false;
+    int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, static_cast<int>(threads), 0) !=
-            cudaSuccess) {
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    if (blocks > static_cast<uint32_t>(sms) * static_cast<uint32_t>(per_sm)) return false;
-    if (blocks_out) *blocks_out = blocks;
-    return true;
+    const bool narrow = run->cfg.tournament_size == 5u && run->cfg.model == GA_MODEL_TRAIT;
+    const uint32_t per_sm = N == 32u ? 40u : N == 64u ? (narrow ? 36u : 32u) : kResidentMaxIslands;
+    return run->n_islands <= static_cast<uint64_t>(sms) * per_sm;
 }
 
-cudaError_t launch_resident(ga_run *run, const void *src, void *dst, uint32_t g0, uint32_t n_gens,
-                            cudaStream_t stream)
+// A streamed launch covers a migration interval of k generations, so resident launches save
+// k - 1 launches less as k grows, while the streamed kernels keep twice the warps on an SM.  Us
+// per generation, streamed / resident, on either side of each line:
+//   k = 1   N = 32: 1.0M agents 10.3 / 7.9, 2.0M 14.4 / 13.3;  N = 16: 0.8M 10.2 / 7.5, 1.0M 10.3 / 10.6
+//   k = 2   N = 32: 1.3M 9.3 / 9.3, 1.6M 10.3 / 10.9;  N = 8: 262,000 3.1 / 2.8, 400,000 4.2 / 4.3
+//   k = 4   N = 32: 400,000 3.7 / 2.7, 600,000 3.7 / 4.0;  N = 16: 262,000 2.6 / 2.2, 400,000 3.1 / 3.2;
+//           48-byte records, N = 32: 131,000 2.1 / 1.4, 600,000 4.2 / 4.5
+//   k = 16  N = 32: 400,000 2.8 / 2.6, 600,000 2.8 / 3.8;  N = 16: 65,000 1.2 / 0.7, 262,000 1.5 / 2.0;
+//           N = 8 and wider records: 65,000 0.57 / 0.65 and 0.69 / 0.69
+bool resident_pays(const ga_run *run)
 {
-    uint32_t threads = 0, per_block = 0;
-    const ResidentKernel k =
-        pick_resident(run->cfg.island_size, run->cfg.model, run->cfg.tournament_size, threads, per_block);
-    if (!k) return cudaErrorInvalidValue;
-    const uint32_t blocks = (run->n_islands + per_block - 1) / per_block;
-    // empty mailboxes (all ones) and a clear abort word for this launch
-    uint8_t *state = static_cast<uint8_t *>(run->resident_state);
-    cudaError_t e = cudaMemsetAsync(state, 0, 256, stream);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(state + 256, 0xFF, static_cast<size_t>(run->n_islands) * 4u * 2u * 16u, stream);
-    if (e != cudaSuccess) return e;
+    const uint32_t k = run->per_neighbor ? run->every_k : 0xFFFFFFFFu;
+    const uint32_t N = run->cfg.island_size;
+    if (k == 1u) return run->n_islands <= 65536u;
+    if (k == 2u) return run->n_islands <= 40000u;
+    if (N == 8u || run->record_bytes != 16u) return k <= 8u && run->n_agents <= 131072u;
+    if (N == 16u) return run->n_agents <= (k <= 8u ? 262144u : 131072u);
+    return run->n_agents <= 400000u;
+}
+
+bool resident_plan(const ga_run *run, ResidentPlan &plan)
+{
+    if (run->cfg.mode != GA_SYNC || !run->counters_uniform) return false;
+    const ResidentPick m = pick(run);
+    if (!m.k) return false;
+    int dev = 0, sms = 0, smem = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(reinterpret_cast<const void *>(m.k),
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (static_cast<uint64_t>(run->n_islands) * m.bytes_per_island > static_cast<uint64_t>(sms) * smem) return false;
+    // as few islands per warp as the device holds at once: more warps hide the mailbox trips
+    const uint32_t n_units = (run->n_islands + m.islands_per_unit - 1u) / m.islands_per_unit;
+    for (uint32_t units = 1;; ++units) {
+        const uint32_t per_block = kWarps * units;
+        const size_t bytes = static_cast<size_t>(per_block) * m.islands_per_unit * m.bytes_per_island;
+        if (bytes > static_cast<size_t>(smem)) return false;
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, m.k, kWarps * 32, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        const uint32_t blocks = (n_units + per_block - 1u) / per_block;
+        if (blocks <= static_cast<uint32_t>(sms) * static_cast<uint32_t>(per_sm)) {
+            plan.units = units;
+            plan.blocks = blocks;
+            plan.shared_bytes = bytes;
+            return true;
+        }
+    }
+}
+
+cudaError_t launch_resident(ga_run *run, const ResidentPlan &plan, const void *src, void *dst, uint32_t g0,
+                            uint32_t n_gens, cudaStream_t stream)
+{
+    const ResidentPick m = pick(run);
+    if (!m.k) return cudaErrorInvalidValue;
     ResidentArgs a;
     a.r = run_params(run, src, dst, g0, n_gens, false);
     a.rk = round_keys(Key{static_cast<uint32_t>(run->cfg.seed), static_cast<uint32_t>(run->cfg.seed >> 32)});
-    a.mail = reinterpret_cast<uint4 *>(state + 256);
-    a.abort_word = reinterpret_cast<uint32_t *>(state);
+    if (run->resident_state) {
+        a.mail = reinterpret_cast<uint4 *>(static_cast<uint8_t *>(run->resident_state) + 256);
+        a.mail_stride = m.boxes;
+    } else {
+        a.mail = static_cast<uint4 *>(dst);
+        a.mail_stride = run->cfg.island_size * run->record_bytes / 16u;
+    }
+    a.abort_word = run->d_abort;
     a.wait_ns = static_cast<unsigned long long>(run->resident_wait_us) * 1000ull;
     a.every_k = run->every_k;
     a.per_neighbor = run->per_neighbor;
     a.drop_island = run->drop_island;
+    a.units = plan.units;
+    const uint32_t entries = run->n_islands * m.boxes > n_gens ? run->n_islands * m.boxes : n_gens;
+    const uint32_t blocks = (entries + 255u) / 256u;
+    resident_init_kernel<<<blocks < 1216u ? blocks : 1216u, 256, 0, stream>>>(
+        a.mail, run->n_islands, a.mail_stride, m.boxes, a.abort_word, run->cfg.curation, run->log2_sites,
+        run->cfg.surface_sites, g0, n_gens, run->d_sites, run->cfg.differentia_bits,
+        run->surface_words <= 2u ? run->d_masks : nullptr);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    run->launches += 1;
     void *args[] = {&a};
-    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k), dim3(blocks), dim3(threads),
-                                    args, 0, stream);
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(m.k), dim3(plan.blocks), dim3(kWarps * 32),
+                                    args, plan.shared_bytes, stream);
     run->launches += 1;
     return e;
 }

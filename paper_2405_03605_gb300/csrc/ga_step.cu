@@ -73,15 +73,8 @@ __global__ void curation_sites_kernel(uint32_t policy, uint32_t log2_sites, uint
                                       uint32_t bits, uint2 *__restrict__ masks)
 {
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += gridDim.x * blockDim.x) {
-        const int site = curation_site(policy, log2_sites, sites, t0 + i);
-        out[i] = site;
-        if (masks) {  // sites * bits <= 64: the deposit's bits within surface words 0 and 1
-            const uint32_t pos = site >= 0 ? static_cast<uint32_t>(site) * bits : 0u;
-            const uint32_t m = site >= 0 ? ((1u << bits) - 1u) << (pos & 31u) : 0u;
-            masks[i] = make_uint2(pos < 32u ? m : 0u, pos < 32u ? 0u : m);
-        }
-    }
+         i += gridDim.x * blockDim.x)
+        store_curation_site(policy, log2_sites, sites, t0 + i, bits, &out[i], masks ? &masks[i] : nullptr);
 }
 
 namespace {

@@ -135,3 +135,69 @@ def test_lost_migrants_time_out_and_the_run_recovers():
     o = oracle_for(shape)
     o.step(200)
     assert_same(g.snapshot(), o.snapshot(), 32)
+
+
+@pytest.mark.parametrize("N,rows,cols,S,b,every,tsize,gens", [
+    (32, 91, 101, 64, 1, 1, 5, 60),   # 9,191 islands: several per warp, mailboxes in the population
+    (16, 95, 97, 64, 1, 2, 3, 61),
+    (8, 93, 95, 64, 1, 1, 5, 40),     # the mailboxes fill an island's records exactly
+    (64, 61, 97, 64, 1, 1, 5, 40),
+    (32, 9, 11, 256, 1, 1, 5, 300),   # 48-byte records, deposits in every word
+    (32, 3, 5, 128, 1, 1, 4, 150),    # 32-byte records
+    (16, 5, 7, 32, 8, 2, 5, 90),
+    (64, 4, 9, 128, 1, 4, 5, 90),
+    (8, 6, 7, 256, 1, 1, 5, 90),
+    (16, 13, 1, 128, 1, 1, 8, 50),    # one column: islands their own neighbours
+    (64, 1, 1, 256, 1, 1, 5, 50),
+    (32, 1, 2, 256, 1, 1, 5, 5),
+])
+def test_auto_shapes_match_oracle(N, rows, cols, S, b, every, tsize, gens):
+    """Runs that GA_RESIDENT_AUTO steps resident though they have no mailboxes in their workspace
+    (wider records, more than 8,192 islands): ragged tori, every island and record size, against
+    the oracle; one founder, one set-up and one resident launch each."""
+    shape = RunShape(rows=rows, cols=cols, island_size=N, tournament_size=tsize, surface_sites=S,
+                     differentia_bits=b, migrate_every=every, seed=700 + N + S, run_id=rows, p_ben=0.05,
+                     p_del=0.05)
+    g = _run(shape, gens, RESIDENT_AUTO)
+    assert g.launches == 3
+    o = oracle_for(shape)
+    o.step(gens)
+    assert_same(g.snapshot(), o.snapshot(), N)
+
+
+def test_auto_float_model_split_steps_and_capture():
+    """The float model on 9,180 islands, in calls of odd lengths; the same run captured into a
+    graph; and two such runs stepping on two streams at once."""
+    import torch
+    shape = RunShape(rows=90, cols=102, model=MODEL_FITNESS, p_del=0.33, p_ben=0.003, seed=23)
+    ref = _run(shape, 60, RESIDENT_OFF).snapshot()
+    assert_same(_run(shape, 60, RESIDENT_AUTO, chunks=[1, 7, 4, 48]).snapshot(), ref, 32)
+    from paper_2405_03605_gb300 import ga
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    runs = [ga.Run(shape, stream=s) for s in streams]
+    for _ in range(3):
+        for r in runs:
+            r.step(20)
+    for r in runs:
+        r.sync()
+        assert_same(r.snapshot(), ref, 32)
+    runs[0].reset()
+    runs[0].sync()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=streams[0]):
+        runs[0].step(60)
+    graph.replay()
+    torch.cuda.synchronize()
+    runs[0].sync()
+    assert_same(runs[0].snapshot(), ref, 32)
+
+
+def test_auto_lost_migrants_stream_large_runs():
+    """Fault injection concerns the runs that GA_RESIDENT_ON accepts: a larger run streams with it
+    set, and steps exactly."""
+    shape = RunShape(rows=92, cols=100, seed=29)
+    g = gpu_run(shape)
+    g.inject_lost_migrants(5)
+    g.step(30)
+    g.sync()
+    assert_same(g.snapshot(), _run(shape, 30, RESIDENT_OFF).snapshot(), 32)
