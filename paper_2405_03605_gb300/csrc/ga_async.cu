@@ -176,6 +176,7 @@ island_async_kernel(const AsyncArgs a)
     constexpr int MB = box_words(Q);
     const RunParams &p = a.r;
 
+    wait_previous_grid();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t seg_lane = lane % SEG;
     const uint32_t island =
@@ -416,6 +417,7 @@ __global__ void __launch_bounds__(kAsyncThreads) island_async_gen_kernel(const A
     const RunParams &p = a.r;
     const uint32_t g = p.g0;
 
+    wait_previous_grid();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t seg_lane = lane % SEG;
     const uint32_t local = (threadIdx.x >> 5) * P + lane / SEG;
@@ -651,9 +653,8 @@ cudaError_t launch_island_async(ga_run *run, const void *src, void *dst, uint32_
     const uint32_t N = run->cfg.island_size;
     const uint32_t per_block = kAsyncWarps * (N >= 32 ? 1u : 32u / N);
     const uint32_t blocks = (last - first + per_block - 1) / per_block;
-    k<<<blocks, kAsyncThreads, 0, stream>>>(a);
     run->launches += 1;
-    return cudaGetLastError();
+    return launch_dependent(k, blocks, kAsyncThreads, stream, a);
 }
 
 // ga_step in the asynchronous modes: windows of async_window generations (cut also at the

@@ -436,6 +436,7 @@ __global__ void resident_init_kernel(uint4 *__restrict__ mail, uint32_t n_island
                                      uint32_t log2_sites, uint32_t sites, uint32_t t0, uint32_t count,
                                      int32_t *__restrict__ out, uint32_t bits, uint2 *__restrict__ masks)
 {
+    wait_previous_grid();
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, all = gridDim.x * blockDim.x;
     if (t == 0u) *abort_word = 0u;
     for (uint32_t i = t; i < count; i += all)
@@ -549,11 +550,10 @@ cudaError_t launch_resident(ga_run *run, const ResidentPlan &plan, const void *s
     a.units = plan.units;
     const uint32_t entries = run->n_islands * m.boxes > n_gens ? run->n_islands * m.boxes : n_gens;
     const uint32_t blocks = (entries + 255u) / 256u;
-    resident_init_kernel<<<blocks < 1216u ? blocks : 1216u, 256, 0, stream>>>(
-        a.mail, run->n_islands, a.mail_stride, m.boxes, a.abort_word, run->cfg.curation, run->log2_sites,
-        run->cfg.surface_sites, g0, n_gens, run->d_sites, run->cfg.differentia_bits,
-        run->surface_words <= 2u ? run->d_masks : nullptr);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_dependent(
+        resident_init_kernel, blocks < 1216u ? blocks : 1216u, 256, stream, a.mail, run->n_islands,
+        a.mail_stride, m.boxes, a.abort_word, run->cfg.curation, run->log2_sites, run->cfg.surface_sites, g0,
+        n_gens, run->d_sites, run->cfg.differentia_bits, run->surface_words <= 2u ? run->d_masks : nullptr);
     if (e != cudaSuccess) return e;
     run->launches += 1;
     void *args[] = {&a};

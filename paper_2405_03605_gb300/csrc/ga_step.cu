@@ -18,6 +18,7 @@ struct StepArgs {
 template <int N, int SW, int TS, int MODEL = 0, int CF = 1>
 __global__ void __launch_bounds__(kStepThreads) island_step_kernel(const StepArgs a)
 {
+    wait_previous_grid();
     step_block<N, SW, TS, kStepWarps, MODEL, CF>(a.r, a.rk, blockIdx.x);
 }
 
@@ -32,6 +33,7 @@ constexpr int units_min_blocks() { return N >= 64 ? 6 : 8; }
 template <int N, int TS, int MODEL>
 __global__ void __launch_bounds__(kStepThreads, units_min_blocks<N>()) island_units_kernel(const StepArgs a)
 {
+    wait_previous_grid();
     step_units<N, TS, units_per_block<N>(), MODEL>(a.r, a.rk, blockIdx.x);
 }
 
@@ -42,6 +44,7 @@ __global__ void founder_kernel(uint4 *__restrict__ dst, uint32_t n_agents, uint3
                                uint32_t run_id)
 {
     __shared__ uint32_t words[12];
+    wait_previous_grid();
     if (threadIdx.x < 12) {
         uint32_t val = 0u;
         const uint32_t k = threadIdx.x;
@@ -72,6 +75,7 @@ __global__ void curation_sites_kernel(uint32_t policy, uint32_t log2_sites, uint
                                       uint32_t t0, uint32_t count, int32_t *__restrict__ out,
                                       uint32_t bits, uint2 *__restrict__ masks)
 {
+    wait_previous_grid();
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += gridDim.x * blockDim.x)
         store_curation_site(policy, log2_sites, sites, t0 + i, bits, &out[i], masks ? &masks[i] : nullptr);
@@ -235,10 +239,10 @@ cudaError_t launch_founder(ga_run *run, void *dst)
     const size_t cap = static_cast<size_t>(sm_count()) * 8;
     if (blocks > cap) blocks = cap;
     if (blocks == 0) blocks = 1;
-    founder_kernel<<<static_cast<unsigned>(blocks), 256, 0, run->stream>>>(
-        static_cast<uint4 *>(dst), run->n_agents, q, run->surface_words, top, key, run->cfg.run_id);
     run->launches += 1;
-    return cudaGetLastError();
+    return launch_dependent(founder_kernel, static_cast<unsigned>(blocks), 256, run->stream,
+                            static_cast<uint4 *>(dst), run->n_agents, q, run->surface_words, top, key,
+                            run->cfg.run_id);
 }
 
 cudaError_t launch_counter_check(ga_run *run, uint32_t generation, int *d_flag)
@@ -288,9 +292,8 @@ cudaError_t launch_island_step(ga_run *run, const void *src, void *dst, uint32_t
             a.rk = round_keys(Key{static_cast<uint32_t>(run->cfg.seed),
                                   static_cast<uint32_t>(run->cfg.seed >> 32)});
             const uint32_t blocks = (run->n_islands + islands_per_block - 1) / islands_per_block;
-            ku<<<blocks, kStepThreads, 0, stream>>>(a);
             run->launches += 1;
-            return cudaGetLastError();
+            return launch_dependent(ku, blocks, kStepThreads, stream, a);
         }
     }
     StepKernel k =
@@ -306,9 +309,8 @@ cudaError_t launch_island_step(ga_run *run, const void *src, void *dst, uint32_t
     const uint32_t N = run->cfg.island_size;
     const uint32_t islands_per_block = kStepWarps * (N >= 32 ? 1u : 32u / N);
     const uint32_t blocks = (run->n_islands + islands_per_block - 1) / islands_per_block;
-    k<<<blocks, kStepThreads, 0, stream>>>(a);
     run->launches += 1;
-    return cudaGetLastError();
+    return launch_dependent(k, blocks, kStepThreads, stream, a);
 }
 
 cudaError_t launch_site_table(ga_run *run, uint32_t g0, uint32_t count, cudaStream_t stream)
@@ -330,9 +332,8 @@ cudaError_t launch_curation_sites(uint32_t policy, uint32_t sites, uint32_t t0, 
     while ((1u << s) < sites) ++s;
     uint32_t blocks = (count + 255u) / 256u;
     if (blocks > 8192u) blocks = 8192u;
-    curation_sites_kernel<<<blocks, 256, 0, stream>>>(policy, s, sites, t0, count, d_sites, bits,
-                                                      d_masks);
-    return cudaGetLastError();
+    return launch_dependent(curation_sites_kernel, blocks, 256, stream, policy, s, sites, t0, count, d_sites,
+                            bits, d_masks);
 }
 
 }  // namespace ga
