@@ -10,8 +10,8 @@
 // 8 to 64 agents.  Results are bit-identical to the streamed kernels: the same draws, landing
 // slots, tournaments, mutations and deposits.
 //
-// Mapping: each warp holds a few consecutive islands (units of Shape<N>::P) in shared memory
-// for the whole launch and works through them one unit at a time, as step_units does.  The
+// Mapping: each warp, a block of its own, holds a few consecutive islands (units of Shape<N>::P)
+// in shared memory for the whole launch and works through them one unit at a time.  The
 // migration bookkeeping is done for all the warp's islands at once, one (island, direction)
 // pair per lane.  On a migration generation g the warp
 //   1. pushes: lane (I, d) writes the member that the neighbour in direction d draws into that
@@ -20,7 +20,6 @@
 //      depend on no state) and its first islands' births;
 //   3. polls: lane (I, d) reads I's mailbox for direction d until it holds generation g;
 //   4. lands the arrivals in its islands' records (shared memory) and reproduces.
-// Warps never wait for one another inside a block, and there is no block barrier.
 //
 // Mailboxes: a 16-byte record is its own ready flag (its counter is g); wider records travel as
 // three 16-byte chunks of three words and the generation, their counter being g.  Each chunk is
@@ -39,12 +38,13 @@
 // generation.  The population is then undefined; the status is returned by the next ga_sync.
 //
 // What bounds it: small runs the two L2 trips of a migration (32x32 torus of 32-agent islands:
-// 1.23 us per generation), larger ones issue (9,991 islands of 32: 192 warp-instructions per
-// island and generation at 56% issue, 2.8 us per generation, 7.2 us with one launch each).
-// Per generation, launches before and now: 262,000 agents 6.2 and 2.7 us, 600,000 6.5 and 4.8,
-// 1,000,000 10.3 and 7.4; 48-byte records 33,000 4.2 and 1.6, 262,000 8.3 and 3.2, 600,000
-// 12.8 and 6.2.  48 or 40 registers instead of 64 (more warps, fewer islands each) are slower
-// throughout: 718 and 734 us against 710 us for 250 generations of 9,991 islands.
+// 1.15 us per generation), larger ones issue (9,991 islands of 32: 2.65 us per generation; 7.2 us
+// with one ordinary launch each, 4 with dependent ones).  Shapes, us for 250 generations of 9,991
+// islands of 16-byte and 5,893 of 48-byte records: one warp per block 665 and 562, four 707 and
+// 612 (what depends on the block alone stays in uniform registers); about 18 warps on an SM at
+// up to 96 registers against as many as 64 registers allow: 131,000 agents 1.7 and 2.3 us per
+// generation (the bookkeeping of one island takes a quarter of a warp's lanes), 262,000 2.4 and
+// 2.9.
 #include "ga_device.cuh"
 #include "ga_internal.h"
 #include "ga_island.cuh"
@@ -56,7 +56,9 @@ RunParams run_params(const ga_run *run, const void *src, void *dst, uint32_t g0,
 
 namespace {
 
-constexpr uint32_t kWarps = 4;  // per block
+
+// Warps per SM that a run is spread over, while its islands per warp allow it.
+constexpr uint32_t kWarpsPerSm = 18;
 
 struct ResidentArgs {
     RunParams r;
@@ -131,25 +133,25 @@ __host__ __device__ constexpr uint32_t warp_bytes(uint32_t islands)
     return islands * (N * Record<SW>::Q * 16u + 4u * (4u + 2u + 1u) + 4u);
 }
 
-template <int N, int SW, int TS, int MODEL>
-__global__ void __launch_bounds__(kWarps * 32, 8) resident_kernel(const ResidentArgs a)
+// N, SW, TS, MODEL: island size, surface words, tournament size (0: read from the run) and genome
+// model, as in step_block; IV: migrations more than a generation apart.
+template <int N, int SW, int TS, int MODEL, bool IV>
+__global__ void __launch_bounds__(32, 20) resident_kernel(const ResidentArgs a)
 {
     constexpr int A = Shape<N>::A, P = Shape<N>::P, SEG = Shape<N>::SEG;
     constexpr int LW = Record<SW>::LW, Q = Record<SW>::Q, C = Record<SW>::C;
     extern __shared__ uint4 s_all[];
     const RunParams &p = a.r;
-    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+    const uint32_t lane = threadIdx.x;  // one warp per block
     const uint32_t seg_lane = lane % SEG;
     const uint32_t per_warp = a.units * P;
-    const uint32_t first = (blockIdx.x * kWarps + warp) * per_warp;
-    if (first >= p.n_islands) return;  // whole warps
+    const uint32_t first = blockIdx.x * per_warp;
     const uint32_t count = min(per_warp, p.n_islands - first);
     const uint32_t pairs = count * 4u;  // (island, direction) pairs of the warp
     const uint32_t end = p.g0 + p.n_gens;
 
-    uint8_t *mine = reinterpret_cast<uint8_t *>(s_all) + warp * warp_bytes<N, SW>(per_warp);
-    uint4 *recs = reinterpret_cast<uint4 *>(mine);
-    uint32_t *s_nb = reinterpret_cast<uint32_t *>(mine + per_warp * (N * Q * 16u));
+    uint4 *recs = s_all;
+    uint32_t *s_nb = reinterpret_cast<uint32_t *>(recs + per_warp * (N * Q));
     uint8_t *s_slot = reinterpret_cast<uint8_t *>(s_nb + per_warp * 4u);  // [2][per_warp * 4]
     uint8_t *s_e = s_slot + per_warp * 8u;
 
@@ -216,7 +218,7 @@ __global__ void __launch_bounds__(kWarps * 32, 8) resident_kernel(const Resident
     cp_async_wait<0>();
     __syncwarp();
     bool aborted = false;
-    for (uint32_t it = 0; it < p.n_gens; ++it) {
+    for (uint32_t it = 0, len = 0; it < p.n_gens; it += len) {
         const uint32_t g = p.g0 + it;
         uint2 dm = make_uint2(0u, 0u);
         int site = -1;
@@ -316,6 +318,10 @@ __global__ void __launch_bounds__(kWarps * 32, 8) resident_kernel(const Resident
             gm = gm_next;
         }
         else island_draws<N>(w, sd, a.rk, first + lane / SEG);
+        // IV (16-byte records, migrations more than a generation apart): the generations up to the
+        // next migration in registers (16,384 agents, one migration in 16: 0.31 us per generation,
+        // 0.42 with the records stored and loaded in each)
+        len = IV ? (gm != ~0u ? gm : end) - g : 1u;
         uint4 *own = recs + lane * Q;
         for (uint32_t u = 0; u < count; u += P, own += 32u * A * Q) {
             const uint32_t li = u + lane / SEG;
@@ -337,11 +343,19 @@ __global__ void __launch_bounds__(kWarps * 32, 8) resident_kernel(const Resident
                     for (int k = 0; k < 4; ++k)
                         if (4 * q + k < LW) rec[ag][4 * q + k] = w4[k];
                 }
-            // records wider than 16 bytes take the deposit in shared memory, below
-            if constexpr (SW == 2)
+            // wider records take the deposit in shared memory, below
+            if constexpr (SW == 2) {
                 reproduce<N, SW, TS, MODEL, 0, 1>(rec, w, p, a.rk, island, seg_lane, mask, g, 0, dm);
-            else
+                if constexpr (IV) {
+                    for (uint32_t j = 1; j < len; ++j) {
+                        const uint2 dj = gen_mask_at(p, it + j);
+                        birth_draws<N>(w, p, a.rk, g + j, island, seg_lane);
+                        reproduce<N, SW, TS, MODEL, 0, 1>(rec, w, p, a.rk, island, seg_lane, mask, g + j, 0, dj);
+                    }
+                }
+            } else {
                 reproduce<N, SW, TS, MODEL, 0, 0>(rec, w, p, a.rk, island, seg_lane, mask, g, -1);
+            }
 #pragma unroll
             for (int ag = 0; ag < A; ++ag)
 #pragma unroll
@@ -394,37 +408,44 @@ ResidentPick picked(ResidentKernel k)
 
 // Tournament size 5 (the paper's) is compiled in; other sizes are read from the run.
 template <int N, int SW, int MODEL = 0>
-ResidentPick pick_ts(uint32_t tsize)
+ResidentPick pick_ts(uint32_t tsize, bool intervals)
 {
-    return picked<N, SW>(tsize == 5u ? resident_kernel<N, SW, 5, MODEL> : resident_kernel<N, SW, 0, MODEL>);
+    if constexpr (SW == 2) {
+        if (intervals)
+            return picked<N, SW>(tsize == 5u ? resident_kernel<N, SW, 5, MODEL, true>
+                                             : resident_kernel<N, SW, 0, MODEL, true>);
+    }
+    return picked<N, SW>(tsize == 5u ? resident_kernel<N, SW, 5, MODEL, false>
+                                     : resident_kernel<N, SW, 0, MODEL, false>);
 }
 
 // The float-fitness model: 16-byte records, islands of 16 to 64 agents.  32-byte records: not
 // for islands of 8, whose mailboxes would not fit in the place of their records.
 template <int N>
-ResidentPick pick_n(uint32_t surface_words, uint32_t model, uint32_t tsize)
+ResidentPick pick_n(uint32_t surface_words, uint32_t model, uint32_t tsize, bool intervals)
 {
     if (model == GA_MODEL_FITNESS) {
         if constexpr (N >= 16)
-            if (surface_words <= 2u) return pick_ts<N, 2, 1>(tsize);
+            if (surface_words <= 2u) return pick_ts<N, 2, 1>(tsize, intervals);
         return ResidentPick();
     }
-    if (surface_words <= 2u) return pick_ts<N, 2>(tsize);
+    if (surface_words <= 2u) return pick_ts<N, 2>(tsize, intervals);
     if (surface_words <= 6u) {
-        if constexpr (N >= 16) return pick_ts<N, 6>(tsize);
+        if constexpr (N >= 16) return pick_ts<N, 6>(tsize, intervals);
         return ResidentPick();
     }
-    return pick_ts<N, 8>(tsize);
+    return pick_ts<N, 8>(tsize, intervals);
 }
 
 ResidentPick pick(const ga_run *run)
 {
     const uint32_t sw = run->surface_words, model = run->cfg.model, ts = run->cfg.tournament_size;
+    const bool iv = run->per_neighbor == 0u || run->every_k > 1u;
     switch (run->cfg.island_size) {
-    case 8: return pick_n<8>(sw, model, ts);
-    case 16: return pick_n<16>(sw, model, ts);
-    case 32: return pick_n<32>(sw, model, ts);
-    case 64: return pick_n<64>(sw, model, ts);
+    case 8: return pick_n<8>(sw, model, ts, iv);
+    case 16: return pick_n<16>(sw, model, ts, iv);
+    case 32: return pick_n<32>(sw, model, ts, iv);
+    case 64: return pick_n<64>(sw, model, ts, iv);
     default: return ResidentPick();
     }
 }
@@ -472,23 +493,30 @@ bool resident_eligible(const ga_run *run)
 }
 
 // A streamed launch covers a migration interval of k generations, so resident launches save
-// k - 1 launches less as k grows, while the streamed kernels keep twice the warps on an SM.  Us
-// per generation, streamed / resident, on either side of each line:
-//   k = 1   N = 32: 1.0M agents 10.3 / 7.9, 2.0M 14.4 / 13.3;  N = 16: 0.8M 10.2 / 7.5, 1.0M 10.3 / 10.6
-//   k = 2   N = 32: 1.3M 9.3 / 9.3, 1.6M 10.3 / 10.9;  N = 8: 262,000 3.1 / 2.8, 400,000 4.2 / 4.3
-//   k = 4   N = 32: 400,000 3.7 / 2.7, 600,000 3.7 / 4.0;  N = 16: 262,000 2.6 / 2.2, 400,000 3.1 / 3.2;
-//           48-byte records, N = 32: 131,000 2.1 / 1.4, 600,000 4.2 / 4.5
-//   k = 16  N = 32: 400,000 2.8 / 2.6, 600,000 2.8 / 3.8;  N = 16: 65,000 1.2 / 0.7, 262,000 1.5 / 2.0;
-//           N = 8 and wider records: 65,000 0.57 / 0.65 and 0.69 / 0.69
+// fewer launches as k grows, while the streamed kernels keep three times the warps on an SM.  Us
+// per generation, streamed / resident, on either side of each line (16-byte records but for W,
+// 48-byte ones, and X, 32-byte ones; thousands of agents):
+//   k = 1   N = 8: 131 2.40 / 2.21, 196 3.25 / 3.33;  16: 320 4.3 / 3.4, 400 4.4 / 4.7;
+//           32: 1,300 8.9 / 8.5, 1,600 10.3 / 10.9;  64: 1,300 12.2 / 9.9, 1,600 12.2 / 12.7
+//   k = 2   8: 98 1.37 / 1.35, 131 1.53 / 1.56;  16: 262 2.5 / 2.4, 400 3.2 / 3.9;
+//           32: 500 3.9 / 3.6, 600 3.9 / 4.1;  64: 1,300 10.7 / 10.0, 1,600 10.8 / 12.5;
+//           X: 600 4.4 / 4.3, 800 5.6 / 6.0
+//   k = 4   8: 65 0.78 / 0.72, 98 0.92 / 0.94;  16: 196 1.86 / 1.55, 262 1.88 / 1.99;
+//           32: 400 3.2 / 2.7, 500 3.2 / 3.2;  64: 600 4.3 / 3.9, 1,000 6.7 / 7.8;
+//           W: 196 1.59 / 1.49, 400 2.7 / 2.8;  X: 131 1.14 / 1.15
+//   k = 16  8: 16 0.34 / 0.32, 65 0.44 / 0.51;  16: 196 1.4 / 1.3, 262 1.4 / 1.7;
+//           32: 400 2.7 / 2.4, 500 2.7 / 2.9;  64: 400 3.7 / 3.3, 500 3.7 / 3.8;
+//           W: 16 0.38 / 0.41
 bool resident_pays(const ga_run *run)
 {
     const uint32_t k = run->per_neighbor ? run->every_k : 0xFFFFFFFFu;
-    const uint32_t N = run->cfg.island_size;
-    if (k == 1u) return run->n_islands <= 65536u;
-    if (k == 2u) return run->n_islands <= 40000u;
-    if (N == 8u || run->record_bytes != 16u) return k <= 8u && run->n_agents <= 131072u;
-    if (N == 16u) return run->n_agents <= (k <= 8u ? 262144u : 131072u);
-    return run->n_agents <= 400000u;
+    const uint32_t N = run->cfg.island_size, bytes = run->record_bytes;
+    uint32_t most = 0;  // agents
+    if (k == 1u) most = N == 8u ? 150000u : N == 16u && bytes == 16u ? 380000u : 1400000u;
+    else if (k == 2u) most = N == 8u ? 98304u : bytes != 16u ? 600000u : N == 16u ? 300000u : N == 32u ? 500000u : 1400000u;
+    else if (k <= 8u) most = N == 8u ? 65536u : bytes == 32u ? 131072u : bytes == 48u || N == 16u ? 200000u : N == 32u ? 400000u : 600000u;
+    else if (N >= 16u && bytes == 16u) most = N == 16u ? 200000u : 400000u;
+    return run->n_agents <= most;
 }
 
 bool resident_plan(const ga_run *run, ResidentPlan &plan)
@@ -506,18 +534,18 @@ bool resident_plan(const ga_run *run, ResidentPlan &plan)
         return false;
     }
     if (static_cast<uint64_t>(run->n_islands) * m.bytes_per_island > static_cast<uint64_t>(sms) * smem) return false;
-    // as few islands per warp as the device holds at once: more warps hide the mailbox trips
+    // islands per warp for about kWarpsPerSm warps on an SM, more where they don't fit at once
     const uint32_t n_units = (run->n_islands + m.islands_per_unit - 1u) / m.islands_per_unit;
-    for (uint32_t units = 1;; ++units) {
-        const uint32_t per_block = kWarps * units;
-        const size_t bytes = static_cast<size_t>(per_block) * m.islands_per_unit * m.bytes_per_island;
+    const uint32_t want = static_cast<uint32_t>(sms) * kWarpsPerSm;
+    for (uint32_t units = (n_units + want - 1u) / want;; ++units) {
+        const size_t bytes = static_cast<size_t>(units) * m.islands_per_unit * m.bytes_per_island;
         if (bytes > static_cast<size_t>(smem)) return false;
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, m.k, kWarps * 32, bytes) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, m.k, 32, bytes) != cudaSuccess) {
             cudaGetLastError();
             return false;
         }
-        const uint32_t blocks = (n_units + per_block - 1u) / per_block;
+        const uint32_t blocks = (n_units + units - 1u) / units;
         if (blocks <= static_cast<uint32_t>(sms) * static_cast<uint32_t>(per_sm)) {
             plan.units = units;
             plan.blocks = blocks;
@@ -557,7 +585,7 @@ cudaError_t launch_resident(ga_run *run, const ResidentPlan &plan, const void *s
     if (e != cudaSuccess) return e;
     run->launches += 1;
     void *args[] = {&a};
-    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(m.k), dim3(plan.blocks), dim3(kWarps * 32),
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(m.k), dim3(plan.blocks), dim3(32),
                                     args, plan.shared_bytes, stream);
     run->launches += 1;
     return e;
