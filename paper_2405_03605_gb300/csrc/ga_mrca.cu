@@ -1,64 +1,29 @@
 // ga_mrca.cu -- pairwise MRCA bounds over sampled end-state agents (post hoc relatedness
 // estimation from hstrat markers, Fig. 1 caption of the paper).
 //
-// Pipeline (all on the run's stream).  Strings of at most 64 bits (S b <= 64), two launches:
-//   1. pack64_kernel : one thread per sampled agent; each block first finds the ranks the
-//                      surface retains at counter T in closed form (no replay of ranks
-//                      0..T-1: one thread per retained rank or site) and sorts the occupied
-//                      sites by rank, r_0 < ... < r_{m-1} (block 0 also writes them out for
-//                      the pair kernel); each thread then gathers its agent's differentiae in
-//                      rank order into one 64-bit string, stored bit-reversed (the first rank
-//                      index at bit 63), 8 bytes per agent.
-//   2. pair64_kernel : one thread per pair (i, j), j > i, in output order; the count of
-//                      leading zeros of packed[i] ^ packed[j] gives the first mismatching
-//                      rank index i*, from which hi = r_{i*} and lo = r_{i*-K} + 1 (0 if
-//                      i* < K); with no mismatch hi = T, lo = r_{m-K} + 1 (0 if m < K).
-// Wider strings (up to 256 bits), three launches: rank_table_kernel (the same closed form,
-// once), pack_kernel (one warp per agent, 8 words), pair_kernel (the first nonzero word of the
-// XOR, then the same rules).
-// The pair kernels are bound by their output: 8 bytes (lo, hi) per pair, written once with
-// streaming stores.
+// Synchronous runs (one counter T) take two launches, pack_kernel and pair_kernel; asynchronous
+// ones (counters differ) two others, mixed_table_kernel and mixed_pair_kernel (each described
+// there).
 #include "ga_device.cuh"
 #include "ga_internal.h"
+
+#include <type_traits>
 
 namespace ga {
 
 namespace {
 
 constexpr uint32_t kPackWords = 8;  // 256-bit rank-ordered strings
-constexpr int kPairThreads = 256;
-constexpr unsigned long long kPairGrid = 152ull * 8ull;  // 8 resident blocks on each of 152 SMs
-constexpr uint32_t kPack64Threads = 128;  // >= 64 sites; small blocks spread a sample over SMs
-
-
-struct MrcaLayout {
-    uint32_t *order;   // [S]  sites sorted by rank
-    uint32_t *ranks;   // [S]  sorted ranks
-    uint32_t *meta;    // [4]  m
-    uint32_t *packed;  // [n][kPackWords] (strings of at most 64 bits: [n] 64-bit words)
-};
-
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Scratch bytes of one synchronous MRCA call: order, ranks, meta, packed strings.
-size_t sync_scratch_bytes(uint32_t S, uint32_t n)
+// Scratch of a synchronous call: the bounds by first differing bit, then the sampled agents'
+// strings of 2 or 8 words (S b <= 64; up to 256 bits).
+constexpr size_t kTableBytes = 257 * sizeof(uint2) + 248;  // padded to 256 bytes
+static_assert(kTableBytes % 256 == 0, "strings aligned");
+uint32_t string_words(uint32_t sites, uint32_t bits) { return sites * bits <= 64u ? 2u : 8u; }
+size_t sync_scratch_bytes(uint32_t sites, uint32_t bits, uint32_t n)
 {
-    return 2 * align_up(S * 4u, 256) + 256 + static_cast<size_t>(n) * kPackWords * 4u;
-}
-
-MrcaLayout carve(void *scratch, uint32_t S)
-{
-    uint8_t *p = static_cast<uint8_t *>(scratch);
-    MrcaLayout l;
-    size_t off = 0;
-    l.order = reinterpret_cast<uint32_t *>(p + off);
-    off = align_up(off + S * 4u, 256);
-    l.ranks = reinterpret_cast<uint32_t *>(p + off);
-    off = align_up(off + S * 4u, 256);
-    l.meta = reinterpret_cast<uint32_t *>(p + off);
-    off = align_up(off + 16u, 256);
-    l.packed = reinterpret_cast<uint32_t *>(p + off);
-    return l;
+    return kTableBytes + static_cast<size_t>(n) * string_words(sites, bits) * 4u;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -138,85 +103,203 @@ __device__ __forceinline__ uint32_t retained_entry(uint32_t policy, uint32_t s, 
     return r1 ? 2u * r1 : 0u;
 }
 
-// One block of 256 threads: the retained ranks at T placed at their sites (shared memory),
-// then the occupied sites sorted by rank: order[i] = site of the i-th smallest retained rank,
-// ranks[i] = that rank, meta[0] = m.
-__global__ void __launch_bounds__(256)
-rank_table_kernel(uint32_t *__restrict__ order, uint32_t *__restrict__ ranks,
-                  uint32_t *__restrict__ meta, uint32_t policy, uint32_t log2_sites,
-                  uint32_t sites, uint32_t T)
+// 32 x 32 bit transposes across a warp: bit (r, c) -- lane r's bit c -- moves to (c, r), in five
+// exchanges of half-width blocks.  The lane's masks, byte selectors and rotations are made once.
+struct Transpose32 {
+    uint32_t select16, select8, keep[3], turn[3];
+    __device__ __forceinline__ explicit Transpose32(uint32_t lane)
+    {
+        select16 = (lane & 16u) ? 0x3276u : 0x5410u;
+        select8 = (lane & 8u) ? 0x3715u : 0x6240u;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t j = 4u >> k, low = k == 0 ? 0x0F0F0F0Fu : k == 1 ? 0x33333333u : 0x55555555u;
+            keep[k] = (lane & j) ? ~low : low;
+            turn[k] = (lane & j) ? 32u - j : j;
+        }
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t x) const
+    {
+        x = __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 16), select16);
+        x = __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 8), select8);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            uint32_t y = __shfl_xor_sync(0xffffffffu, x, 4 >> k);
+            y = __funnelshift_l(y, y, turn[k]);
+            x = (x & keep[k]) | (y & ~keep[k]);
+        }
+        return x;
+    }
+};
+
+uint32_t margin(uint32_t bits)
 {
-    __shared__ uint32_t h[256];
-    release_next_grid();  // the pack kernel may start loading its agents' records
-    const uint32_t k = threadIdx.x;
-    h[k] = 0u;
+    // smallest K with 2^(-bits*K) < 0.05, i.e. bits*K > log2(20) = 4.32
+    uint32_t K = 1;
+    while (bits * K <= 4u) ++K;
+    return K;
+}
+
+// ---------------------------------------------------------------------------------------
+// One counter T.  With r_0 < ... < r_{m-1} the ranks retained at T and i* the first rank index
+// at which two agents' differentiae differ: hi = r_{i*} and lo = r_{i*-K} + 1 (0 if i* < K);
+// with no mismatch hi = T and lo = r_{m-K} + 1 (0 if m < K).
+//   1. pack_kernel: 256 agents per block.  The rank order at T in closed form, in every block:
+//      thread k < S finds retained entry k and puts it at its site; the occupied sites are sorted
+//      by counting smaller ranks (block 0 writes the table of both bounds by first differing
+//      bit).  Each warp packs 32 agents into strings with differentia index i in bits
+//      [i b, i b + b), each word bit-reversed so that the first differing bit of a pair is the
+//      highest of the first words that differ.  The permutation from site order to rank order
+//      moves bit planes: a 32 x 32 bit transpose turns 32 agents' words into one word per surface
+//      bit, which are read back in rank order and transposed again.  Bound by two dependent reads,
+//      ids and records.
+//   2. pair_kernel: one thread per pair in output order, each warp a contiguous stretch of whole
+//      128-byte lines; lane t takes pairs base + t, base + t + 32, ... and steps 32 columns at a
+//      time, reloading row i's string only when a step carries it into the next rows.  Per pair one
+//      string load (8 bytes; 32 where S b > 64), a find-highest-bit and one table read.  Bound by
+//      the bounds it writes, 8 bytes per pair: a plain fill of the same 67 MB takes 12.5 us.
+// Slower: rows taken whole by a warp, whose ends leave part of a line to the next row (16.5 us
+// for the call of 4,096 agents, 17.8 unrolled by four); 4-byte string and table reads (20.2 us);
+// one launch in which a block packs the agents of its own tile of pairs (17 to 24 us).
+// The call (with the order, now found while the previous grid drains, and the bit-by-bit gather it
+// took 4 us before the pair kernel): 4,096 agents with 64 sites (8.4M pairs) 14.1 us, 18.3 before;
+// 3,000 agents with 256 sites 16.3 us, 28.5 before; 300 agents 5.5 and 7.2 us, 7.9 and 10.7 before.
+// ---------------------------------------------------------------------------------------
+constexpr uint32_t kPairThreads = 256;
+
+// Table entry of a pair: 32 W less the index of the first bit in which its strings of W words
+// differ, 0 for none.  Words are bit-reversed: the first differing bit is the highest of the first
+// words that differ.
+__device__ __forceinline__ uint32_t highest_bit(uint32_t x)
+{
+    uint32_t at;
+    asm("bfind.u32 %0, %1;" : "=r"(at) : "r"(x));  // ~0 for 0
+    return at;
+}
+__device__ __forceinline__ uint32_t pair_entry(uint2 a, uint2 b)
+{
+    const uint32_t x0 = a.x ^ b.x, x1 = a.y ^ b.y;
+    return highest_bit(x0 != 0u ? x0 : x1) + (x0 != 0u ? 33u : 1u);
+}
+struct String8 {
+    uint4 h[2];
+};
+__device__ __forceinline__ uint32_t pair_entry(const String8 &a, const String8 &b)
+{
+    const uint32_t x[8] = {a.h[0].x ^ b.h[0].x, a.h[0].y ^ b.h[0].y, a.h[0].z ^ b.h[0].z, a.h[0].w ^ b.h[0].w,
+                           a.h[1].x ^ b.h[1].x, a.h[1].y ^ b.h[1].y, a.h[1].z ^ b.h[1].z, a.h[1].w ^ b.h[1].w};
+    const bool f = (x[0] | x[1] | x[2] | x[3]) != 0u;
+    const uint32_t y0 = f ? x[0] : x[4], y1 = f ? x[1] : x[5], y2 = f ? x[2] : x[6], y3 = f ? x[3] : x[7];
+    const bool g = (y0 | y1) != 0u;
+    const uint32_t z0 = g ? y0 : y2, z1 = g ? y1 : y3;
+    const bool k = z0 != 0u;
+    return highest_bit(k ? z0 : z1) + 1u + (f ? 128u : 0u) + (g ? 64u : 0u) + (k ? 32u : 0u);
+}
+// The string of sampled agent a of n: W = 2, an 8-byte word each; W = 8, two arrays of 16 bytes.
+__device__ __forceinline__ void read_string(const void *packed, uint32_t, uint32_t a, uint2 &v)
+{
+    v = __ldg(static_cast<const uint2 *>(packed) + a);
+}
+__device__ __forceinline__ void read_string(const void *packed, uint32_t n, uint32_t a, String8 &v)
+{
+    v.h[0] = __ldg(static_cast<const uint4 *>(packed) + a);
+    v.h[1] = __ldg(static_cast<const uint4 *>(packed) + n + a);
+}
+
+// W: words of a string (2: S b <= 64; 8: up to 256 bits).
+template <uint32_t W>
+__global__ void __launch_bounds__(256)
+pack_kernel(const uint4 *__restrict__ pop, uint32_t record_quads, uint32_t n_agents,
+            const uint32_t *__restrict__ ids, uint32_t n, uint32_t policy, uint32_t log2_sites,
+            uint32_t log2_bits, uint32_t K, uint32_t T, uint2 *__restrict__ tab,
+            void *__restrict__ packed, int *__restrict__ status)
+{
+    constexpr uint32_t kEmpty = 0xFFFFFFFFu;          // ranks are below a counter
+    __shared__ __align__(16) uint32_t held[32 * W];  // by site: its rank
+    __shared__ uint32_t rank_s[32 * W], place[32 * W];  // by rank index: rank, site bit
+    __shared__ uint32_t plane[8][32u * W];
+    const uint32_t k = threadIdx.x, warp = k >> 5, lane = k & 31u;
+    const uint32_t a = blockIdx.x * 256u + k;
+    const uint32_t sites = 1u << log2_sites, bits = 1u << log2_bits;
+    const uint32_t words = (sites * bits + 31u) >> 5;
+    // the rank order needs nothing from the grid before
+    if (k < 32u * W) held[k] = kEmpty;
     __syncthreads();
     if (k < sites) {
         uint32_t site = 0;
         const uint32_t r1 = retained_entry(policy, log2_sites, sites, T, k, site);
-        if (r1 != 0u) h[site] = r1;
+        if (r1 != 0u && in_bounds(site < sites, status)) held[site] = r1 - 1u;
     }
     __syncthreads();
-    const uint32_t mine = h[k];
-    const int m = __syncthreads_count(mine != 0u);
-    if (mine != 0u) {
+    const uint32_t mine = k < sites ? held[k] : kEmpty;
+    const uint32_t m = static_cast<uint32_t>(__syncthreads_count(mine != kEmpty));
+    if (mine != kEmpty) {
         uint32_t pos = 0;
-        for (uint32_t q = 0; q < sites; ++q) pos += (h[q] != 0u && h[q] < mine) ? 1u : 0u;
-        order[pos] = k;
-        ranks[pos] = mine - 1u;
+        for (uint32_t q = 0; q < sites; q += 4u) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(&held[q]);
+            pos += (v.x < mine) + (v.y < mine) + (v.z < mine) + (v.w < mine);
+        }
+        rank_s[pos] = mine;
+        place[pos] = k << log2_bits;
     }
-    if (k == 0) meta[0] = static_cast<uint32_t>(m);
-}
-
-// Retained ranks at counter T, sorted (order, ranks, meta[0] = m): one launch for any T.
-cudaError_t launch_rank_table(uint32_t *order, uint32_t *ranks, uint32_t *meta, uint32_t policy,
-                              uint32_t log2_sites, uint32_t sites, uint32_t T, cudaStream_t stream)
-{
-    rank_table_kernel<<<1, 256, 0, stream>>>(order, ranks, meta, policy, log2_sites, sites, T);
-    return cudaGetLastError();
-}
-
-// One warp per sampled agent: lanes 0..7 hold the agent's surface words; for packed word w,
-// lane l gathers differentia index w * (32/b) + l (site order[i], fetched from the lane that
-// holds its surface word) and one warp OR-reduction assembles the word.
-__global__ void pack_kernel(const uint32_t *__restrict__ pop, uint32_t record_words,
-                            uint32_t n_agents, const uint32_t *__restrict__ ids, uint32_t n,
-                            const uint32_t *__restrict__ order, const uint32_t *__restrict__ meta,
-                            uint32_t bits, uint32_t T, uint32_t *__restrict__ packed,
-                            int *__restrict__ status)
-{
-    __shared__ uint32_t ord[256];
-    release_next_grid();  // the pair kernel may start its index set-up
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t a = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    // the agent's record does not depend on the rank order: load it before waiting for it
-    const uint32_t id = a < n ? ids[a] : 0u;
-    const bool ok = a < n && id < n_agents;
-    const uint32_t *rec = pop + static_cast<size_t>(ok ? id : 0u) * record_words;
-    const uint32_t counter = ok ? rec[1] : T;
-    const uint32_t surf = (ok && lane < kPackWords && 2u + lane < record_words) ? rec[2 + lane] : 0u;
+    // the previous grid may still be writing the population (or reading what this call
+    // overwrites); the pair kernel may start its set-up
     wait_previous_grid();
-    const uint32_t m = meta[0];
-    for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) ord[i] = order[i];
-    __syncthreads();
-    if (a >= n) return;  // whole warps
-    uint32_t word_out = 0;
-    if (!ok) {
-        if (lane == 0) atomicCAS(status, GA_OK, GA_EINVAL);
-    } else {
-        if (lane == 0 && counter != T) atomicCAS(status, GA_OK, GA_ESTATE);
-        const uint32_t per = 32u / bits, mask = (1u << bits) - 1u;
-        const uint32_t pw = (m * bits + 31u) >> 5;
-        for (uint32_t w = 0; w < pw; ++w) {
-            const uint32_t i = w * per + lane;
-            const uint32_t pos = (lane < per && i < m) ? ord[i] * bits : 0u;
-            const uint32_t sw = __shfl_sync(0xffffffffu, surf, static_cast<int>(pos >> 5));
-            const uint32_t v = (lane < per && i < m) ? ((sw >> (pos & 31u)) & mask) << (lane * bits) : 0u;
-            const uint32_t full = __reduce_or_sync(0xffffffffu, v);
-            if (lane == w) word_out = full;
+    release_next_grid();
+    uint32_t w[W];
+#pragma unroll
+    for (uint32_t e = 0; e < W; ++e) w[e] = 0u;
+    if (a < n) {
+        const uint32_t id = __ldg(&ids[a]);
+        if (id >= n_agents) {
+            atomicCAS(status, GA_OK, GA_EINVAL);
+        } else {
+            const uint4 *r = pop + static_cast<size_t>(id) * record_quads;
+            const uint4 q0 = __ldg(&r[0]);
+            w[0] = q0.z;
+            w[1] = words > 1u ? q0.w : 0u;
+            if constexpr (W > 2u) {  // records of 32 or 48 bytes
+                const uint4 q1 = __ldg(&r[1]);
+                w[2] = q1.x;
+                w[3] = words > 3u ? q1.y : 0u;
+                w[4] = words > 4u ? q1.z : 0u;
+                w[5] = words > 5u ? q1.w : 0u;
+                if (record_quads > 2u) {
+                    const uint4 q2 = __ldg(&r[2]);
+                    w[6] = words > 6u ? q2.x : 0u;
+                    w[7] = words > 7u ? q2.y : 0u;
+                }
+            }
+            if (q0.y != T) atomicCAS(status, GA_OK, GA_ESTATE);
         }
     }
-    if (lane < kPackWords) packed[static_cast<size_t>(a) * kPackWords + lane] = word_out;
+    __syncthreads();
+    if (blockIdx.x == 0)
+        for (uint32_t c = k; c <= 32u * W; c += 256u) {  // c: first differing bit, 32 W: none
+            const uint32_t r = min(c >> log2_bits, m);
+            tab[32u * W - c] = make_uint2(r >= K ? rank_s[r - K] + 1u : 0u, r < m ? rank_s[r] : T);
+        }
+    if (blockIdx.x * 256u + 32u * warp >= n) return;  // whole warps
+    const Transpose32 transpose(lane);
+#pragma unroll
+    for (uint32_t e = 0; e < W; ++e)
+        if (e < words) plane[warp][32u * e + lane] = transpose(w[e]);
+    __syncwarp();
+#pragma unroll
+    for (uint32_t e = 0; e < W; ++e) {
+        w[e] = 0u;
+        if (e < words) {
+            const uint32_t q = 32u * e + lane, i = q >> log2_bits;
+            w[e] = __brev(transpose(i < m ? plane[warp][place[i] + (q & (bits - 1u))] : 0u));
+        }
+    }
+    if (a >= n) return;
+    if constexpr (W == 2u) {
+        static_cast<uint2 *>(packed)[a] = make_uint2(w[0], w[1]);
+    } else {
+        static_cast<uint4 *>(packed)[a] = make_uint4(w[0], w[1], w[2], w[3]);
+        static_cast<uint4 *>(packed)[static_cast<size_t>(n) + a] = make_uint4(w[4], w[5], w[6], w[7]);
+    }
 }
 
 // Row and column of pair p in output order: row i holds pairs off(i) <= p < off(i + 1) with
@@ -233,113 +316,33 @@ __device__ __forceinline__ void first_pair(uint32_t n, uint32_t p, uint32_t &i, 
     j = i + 1u + static_cast<uint32_t>(p - static_cast<unsigned long long>(i) * (b - i) / 2ull);
 }
 
-// Strings of at most 64 bits: one thread per sampled agent.  Each block first builds the
-// rank order itself (threads k < S: retained entry k in closed form, placed at its site; the
-// occupied sites then sorted by rank), so no launch precedes this one; block 0 also writes the
-// sorted ranks and m for the pair kernel.  Thread a then reads agent ids[a]'s 64-bit surface
-// (differentia at site k in bits [k b, k b + b)) and assembles the string with differentia
-// index i at bits [i b, i b + b), stored bit-reversed: the first rank index at bit 63, so a
-// pair's first mismatch is the count of leading zeros of the XOR.  Bits past m b stay zero.
-__global__ void __launch_bounds__(kPack64Threads)
-pack64_kernel(const uint32_t *__restrict__ pop, uint32_t record_words, uint32_t n_agents,
-              const uint32_t *__restrict__ ids, uint32_t n, uint32_t policy, uint32_t log2_sites,
-              uint32_t sites, uint32_t bits, uint32_t T, uint32_t *__restrict__ ranks,
-              uint32_t *__restrict__ meta, unsigned long long *__restrict__ packed,
-              int *__restrict__ status)
-{
-    __shared__ __align__(16) uint32_t h[64];
-    __shared__ uint32_t shift[64];  // surface bit offset of differentia index i
-    release_next_grid();  // the pair kernel may start its index set-up
-    const uint32_t k = threadIdx.x;
-    const uint32_t a = blockIdx.x * blockDim.x + k;
-    const uint32_t id = a < n ? ids[a] : 0u;
-    const bool ok = a < n && id < n_agents;
-    const uint32_t *rec = pop + static_cast<size_t>(ok ? id : 0u) * record_words;
-    const uint32_t counter = ok ? rec[1] : T;
-    const uint32_t w0 = ok ? rec[2] : 0u;
-    const uint32_t w1 = (ok && record_words > 3u) ? rec[3] : 0u;
-    if (k < 64u) h[k] = 0u;
-    __syncthreads();
-    if (k < sites) {
-        uint32_t site = 0;
-        const uint32_t r1 = retained_entry(policy, log2_sites, sites, T, k, site);
-        if (r1 != 0u && in_bounds(site < sites, status)) h[site] = r1;
-    }
-    __syncthreads();
-    const uint32_t mine = k < sites ? h[k] : 0u;
-    const uint32_t m = static_cast<uint32_t>(__syncthreads_count(mine != 0u));
-    if (mine != 0u) {  // position among the occupied sites, all 64 entries read at once
-        uint32_t pos = 0;
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            const uint4 v = reinterpret_cast<const uint4 *>(h)[q];
-            pos += (v.x != 0u && v.x < mine) + (v.y != 0u && v.y < mine) +
-                   (v.z != 0u && v.z < mine) + (v.w != 0u && v.w < mine);
-        }
-        shift[pos] = k * bits;
-        if (blockIdx.x == 0) ranks[pos] = mine - 1u;
-    }
-    if (blockIdx.x == 0 && k == 0) meta[0] = m;
-    __syncthreads();
-    if (a >= n) return;
-    if (!ok) {
-        atomicCAS(status, GA_OK, GA_EINVAL);
-        packed[a] = 0ull;
-        return;
-    }
-    if (counter != T) atomicCAS(status, GA_OK, GA_ESTATE);
-    // differentia index i goes to bits [i b, i b + b) of (o1 : o0); a differentia never
-    // straddles a surface word (b divides 32)
-    const uint32_t mask = (1u << bits) - 1u;
-    uint32_t o0 = 0u, o1 = 0u;
-#pragma unroll 8
-    for (uint32_t i = 0; i < m; ++i) {
-        const uint32_t sh = shift[i];
-        const uint32_t v = (((sh & 32u) ? w1 : w0) >> (sh & 31u)) & mask;
-        const uint32_t ob = i * bits;
-        if (ob & 32u) o1 |= v << (ob & 31u);
-        else o0 |= v << (ob & 31u);
-    }
-    // bit-reversed 64-bit string: reverse(o1 : o0) = reverse(o0) : reverse(o1)
-    packed[a] = (static_cast<unsigned long long>(__brev(o0)) << 32) | __brev(o1);
-}
-
-// Pairs of 64-bit strings, in output order, each warp a contiguous stretch of them: lane t
-// takes pairs base + t, base + t + 32, ... (the row of its first pair found as in pair_kernel
-// below), steps 32 pairs at a time and reloads row i's string only when a step carries it into
-// the next rows.  tab[c] holds both bounds for a leading-zero count c in [0, 64]:
-// i* = min(c / b, m), tab[c] = (i* >= K ? r_{i*-K} + 1 : 0, i* < m ? r_{i*} : T).
+template <uint32_t W>
 __global__ void __launch_bounds__(kPairThreads)
-pair64_kernel(const unsigned long long *__restrict__ packed, uint32_t n,
-              const uint32_t *__restrict__ ranks_g, const uint32_t *__restrict__ meta,
-              uint32_t log2_bits, uint32_t K, uint32_t T, uint32_t per_warp,
-              uint32_t *__restrict__ lo, uint32_t *__restrict__ hi, int *__restrict__ status)
+pair_kernel(const void *__restrict__ packed, uint32_t n, const uint2 *__restrict__ tab_g,
+            uint32_t per_warp, uint32_t *__restrict__ lo, uint32_t *__restrict__ hi, int *__restrict__ status)
 {
-    __shared__ uint2 tab[65];
-    const uint32_t n_pairs = n * (n - 1u) / 2u;
+    __shared__ uint2 tab[32 * W + 1];
+    // pairs [warp * per_warp, (warp + 1) * per_warp) of n (n - 1) / 2 (fewer than 2^31)
+    const uint32_t n_pairs = static_cast<uint32_t>(static_cast<unsigned long long>(n) * (n - 1u) / 2ull);
     const uint32_t warp = (blockIdx.x * kPairThreads + threadIdx.x) >> 5;
     const unsigned long long w_end = static_cast<unsigned long long>(warp + 1u) * per_warp;
     const uint32_t p_end = w_end < n_pairs ? static_cast<uint32_t>(w_end) : n_pairs;
     const unsigned long long p0 = static_cast<unsigned long long>(warp) * per_warp + (threadIdx.x & 31u);
     const bool active = p0 < p_end;
-    const uint32_t p = active ? static_cast<uint32_t>(p0) : 0u;
+    uint32_t q = active ? static_cast<uint32_t>(p0) : 0u;
     uint32_t i = 0, j = 1;
-    first_pair(n, p, i, j);
+    first_pair(n, q, i, j);
 
-    wait_previous_grid();  // ranks, m and the strings come from pack64_kernel
-    const uint32_t m = meta[0];
-    for (uint32_t c = threadIdx.x; c <= 64u; c += blockDim.x) {
-        uint32_t r = c >> log2_bits;
-        r = r < m ? r : m;
-        tab[c] = make_uint2(r >= K ? ranks_g[r - K] + 1u : 0u, r < m ? ranks_g[r] : T);
-    }
+    wait_previous_grid();  // the table and the strings come from pack_kernel
+    for (uint32_t c = threadIdx.x; c <= 32u * W; c += kPairThreads) tab[c] = tab_g[c];
     __syncthreads();
     if (!active || !in_bounds(i < j && j < n, status)) return;
 
-    unsigned long long row = __ldg(packed + i);
-    for (uint32_t q = p;;) {
-        const unsigned long long x = __ldg(packed + j) ^ row;
-        const uint2 bound = tab[__clzll(static_cast<long long>(x))];  // first differing bit, 64: none
+    std::conditional_t<W == 2u, uint2, String8> row, other;
+    read_string(packed, n, i, row);
+    for (;;) {
+        read_string(packed, n, j, other);
+        const uint2 bound = tab[pair_entry(row, other)];
         __stcs(lo + q, bound.x);
         __stcs(hi + q, bound.y);
         q += 32u;
@@ -351,155 +354,35 @@ pair64_kernel(const unsigned long long *__restrict__ packed, uint32_t n,
                 ++i;
             } while (j >= n);
             if (!in_bounds(i < j, status)) break;
-            row = __ldg(packed + i);
+            read_string(packed, n, i, row);
         }
     }
 }
 
-// Pairs of strings wider than 64 bits, in output order, each warp a contiguous stretch of
-// them: lane t takes pairs base + t, base + t + 32, ..., so a warp's (lo, hi) writes are
-// contiguous.  A lane finds the row of its first pair once (first_pair), then steps 32 pairs
-// at a time, carrying into the next rows when j passes n - 1, and reloads row i's string only
-// when i changes.  Pair indices fit 32 bits (n <= 65536: fewer than 2^31 pairs).  The first
-// set bit of packed[i] ^ packed[j] (the first nonzero word, then its lowest set bit) gives the
-// first mismatching rank index i*.  With 0-based sorted ranks r_0 < ... < r_{m-1}, a mismatch
-// at index i* gives hi = r_{i*}, lo = r_{i*-K} + 1 (0 if i* < K), and no mismatch hi = T,
-// lo = r_{m-K} + 1.
-__global__ void __launch_bounds__(kPairThreads)
-pair_kernel(const uint32_t *__restrict__ packed, uint32_t n, const uint32_t *__restrict__ ranks_g,
-            const uint32_t *__restrict__ meta, uint32_t log2_bits, uint32_t K, uint32_t T,
-            uint32_t per_warp, uint32_t *__restrict__ lo, uint32_t *__restrict__ hi,
-            int *__restrict__ status)
+// Both launches of one synchronous MRCA call (shared by the allocating and the fixed-scratch
+// entry points).
+cudaError_t launch_sync_mrca(const void *pop, uint32_t record_bytes, uint32_t n_agents, const uint32_t *d_ids,
+                             uint32_t n, void *scratch, uint32_t policy, uint32_t log2_sites, uint32_t sites,
+                             uint32_t bits, uint32_t T, uint32_t *d_lo, uint32_t *d_hi, int *status,
+                             cudaStream_t stream)
 {
-    __shared__ uint32_t ranks[256];
-    // pairs [warp * per_warp, (warp + 1) * per_warp) of n (n - 1) / 2 (per_warp: a multiple of
-    // 32 chosen on the host so that the grid covers every pair)
-    const uint32_t n_pairs = n * (n - 1u) / 2u;
-    const uint32_t warp = (blockIdx.x * kPairThreads + threadIdx.x) >> 5;
-    const unsigned long long w_end = static_cast<unsigned long long>(warp + 1u) * per_warp;
-    const uint32_t p_end = w_end < n_pairs ? static_cast<uint32_t>(w_end) : n_pairs;
-    const unsigned long long p0 = static_cast<unsigned long long>(warp) * per_warp + (threadIdx.x & 31u);
-    const bool active = p0 < p_end;
-    const uint32_t p = active ? static_cast<uint32_t>(p0) : 0u;
-    uint32_t i = 0, j = 1;
-    first_pair(n, p, i, j);
-    uint32_t q = p;
-    uint32_t *lo_q = lo + q;
-    uint32_t *hi_q = hi + q;
-
-    // the rank table and the packed strings come from the kernels before this one
-    wait_previous_grid();
-    const uint32_t m = meta[0];
-    for (uint32_t r = threadIdx.x; r < m; r += blockDim.x) ranks[r] = ranks_g[r];
-    __syncthreads();
-    if (!active) return;
-
-    uint32_t row = 0xFFFFFFFFu;  // row whose string a0, a1 hold
-    uint4 a0 = make_uint4(0u, 0u, 0u, 0u), a1 = a0;
-    for (;;) {
-        if (!in_bounds(i < j && j < n, status)) break;
-        if (i != row) {
-            a0 = __ldg(reinterpret_cast<const uint4 *>(packed) + i * (kPackWords / 4u));
-            a1 = __ldg(reinterpret_cast<const uint4 *>(packed) + i * (kPackWords / 4u) + 1u);
-            row = i;
-        }
-        const uint4 b0 = __ldg(reinterpret_cast<const uint4 *>(packed) + j * (kPackWords / 4u));
-        const uint4 b1 = __ldg(reinterpret_cast<const uint4 *>(packed) + j * (kPackWords / 4u) + 1u);
-        const uint32_t x[kPackWords] = {b0.x ^ a0.x, b0.y ^ a0.y, b0.z ^ a0.z, b0.w ^ a0.w,
-                                        b1.x ^ a1.x, b1.y ^ a1.y, b1.z ^ a1.z, b1.w ^ a1.w};
-        uint32_t first_bit = 0xFFFFFFFFu;
-#pragma unroll
-        for (int w = kPackWords - 1; w >= 0; --w)
-            if (x[w] != 0u) first_bit = 32u * w + (__ffs(x[w]) - 1u);
-        uint32_t l, h;
-        if (first_bit == 0xFFFFFFFFu) {
-            h = T;
-            l = m >= K ? ranks[m - K] + 1u : 0u;
-        } else {
-            uint32_t istar = first_bit >> log2_bits;  // first mismatch, 0-based
-            if (!in_bounds(istar < m, status)) istar = 0u;
-            h = ranks[istar];
-            l = istar >= K ? ranks[istar - K] + 1u : 0u;
-        }
-        __stcs(lo_q, l);
-        __stcs(hi_q, h);
-        q += 32u;
-        if (q >= p_end) break;
-        lo_q += 32;
-        hi_q += 32;
-        j += 32u;
-        while (j >= n) {  // past the end of row i: pair (i + 1, i + 2) follows (i, n - 1)
-            j = j - n + i + 2u;
-            ++i;
-        }
-    }
-}
-
-// Grid and stretch length of a pair kernel: enough resident blocks for the whole GPU, each
-// warp then sweeping a contiguous stretch of pairs (a multiple of 32).
-void pair_grid(uint32_t n, uint32_t &grid, uint32_t &per_warp)
-{
-    const unsigned long long pairs = static_cast<unsigned long long>(n) * (n - 1u) / 2ull;
-    const unsigned long long want = (pairs + kPairThreads - 1) / kPairThreads;
-    grid = static_cast<uint32_t>(want < kPairGrid ? want : kPairGrid);
-    const unsigned long long n_warps = static_cast<unsigned long long>(grid) * (kPairThreads / 32);
-    per_warp = static_cast<uint32_t>(((pairs + n_warps - 1ull) / n_warps + 31ull) / 32ull * 32ull);
-}
-
-uint32_t margin(uint32_t bits);
-
-// Every launch of one synchronous MRCA call (shared by the allocating and the fixed-scratch
-// entry points): two for strings of at most 64 bits (pack64, then pair64 as a programmatically
-// dependent launch), three otherwise (rank table, then pack and pair as dependent launches).
-cudaError_t launch_sync_mrca(const uint32_t *pop, uint32_t record_words, uint32_t n_agents,
-                             const uint32_t *d_ids, uint32_t n, const MrcaLayout &l,
-                             uint32_t policy, uint32_t log2_sites, uint32_t sites, uint32_t bits,
-                             uint32_t T, uint32_t *d_lo, uint32_t *d_hi, int *status,
-                             cudaStream_t stream, uint32_t &launches)
-{
-    const uint32_t K = margin(bits);
     const uint32_t log2_bits = bits == 1u ? 0u : bits == 2u ? 1u : bits == 4u ? 2u : 3u;
-    uint32_t grid = 0, per_warp = 0;
-    pair_grid(n, grid, per_warp);
-    unsigned long long *packed64 = reinterpret_cast<unsigned long long *>(l.packed);
-    if (sites * bits <= 64u) {
-        pack64_kernel<<<(n + kPack64Threads - 1u) / kPack64Threads, kPack64Threads, 0, stream>>>(
-            pop, record_words, n_agents, d_ids, n, policy, log2_sites, sites, bits, T, l.ranks,
-            l.meta, packed64, status);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        launches += 1;
-        e = launch_dependent(pair64_kernel, grid, kPairThreads, stream,
-                             static_cast<const unsigned long long *>(packed64), n,
-                             static_cast<const uint32_t *>(l.ranks),
-                             static_cast<const uint32_t *>(l.meta), log2_bits, K, T, per_warp,
-                             d_lo, d_hi, status);
-        if (e == cudaSuccess) launches += 1;
-        return e;
-    }
-    cudaError_t e = launch_rank_table(l.order, l.ranks, l.meta, policy, log2_sites, sites, T, stream);
+    const bool narrow = string_words(sites, bits) == 2u;
+    uint2 *tab = static_cast<uint2 *>(scratch);
+    void *packed = static_cast<uint8_t *>(scratch) + kTableBytes;
+    cudaError_t e = launch_dependent(narrow ? pack_kernel<2> : pack_kernel<8>, (n + 255u) / 256u, 256, stream,
+                                     static_cast<const uint4 *>(pop), record_bytes / 16u, n_agents, d_ids, n,
+                                     policy, log2_sites, log2_bits, margin(bits), T, tab, packed, status);
     if (e != cudaSuccess) return e;
-    launches += 1;
-    e = launch_dependent(pack_kernel, (n + 7u) / 8u, 256, stream, pop, record_words, n_agents,
-                         d_ids, n, static_cast<const uint32_t *>(l.order),
-                         static_cast<const uint32_t *>(l.meta), bits, T, l.packed, status);
-    if (e != cudaSuccess) return e;
-    launches += 1;
-    e = launch_dependent(pair_kernel, grid, kPairThreads, stream,
-                         static_cast<const uint32_t *>(l.packed), n,
-                         static_cast<const uint32_t *>(l.ranks),
-                         static_cast<const uint32_t *>(l.meta), log2_bits, K, T, per_warp, d_lo,
-                         d_hi, status);
-    if (e == cudaSuccess) launches += 1;
-    return e;
-}
-
-uint32_t margin(uint32_t bits)
-{
-    // smallest K with 2^(-bits*K) < 0.05, i.e. bits*K > log2(20) = 4.32
-    uint32_t K = 1;
-    while (bits * K <= 4u) ++K;
-    return K;
+    // enough blocks for the whole GPU (8 resident on each of 152 SMs), each warp then sweeping a
+    // contiguous stretch of whole lines
+    const unsigned long long pairs = static_cast<unsigned long long>(n) * (n - 1u) / 2ull;
+    const unsigned long long want = (pairs + kPairThreads - 1u) / kPairThreads;
+    const uint32_t grid = static_cast<uint32_t>(want < 1216u ? want : 1216u);
+    const unsigned long long warps = static_cast<unsigned long long>(grid) * (kPairThreads / 32u);
+    const uint32_t per_warp = static_cast<uint32_t>(((pairs + warps - 1ull) / warps + 31ull) / 32ull * 32ull);
+    return launch_dependent(narrow ? pair_kernel<2> : pair_kernel<8>, grid, kPairThreads, stream,
+                            static_cast<const void *>(packed), n, static_cast<const uint2 *>(tab), per_warp, d_lo, d_hi, status);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -601,24 +484,6 @@ mixed_table_kernel(const uint32_t *__restrict__ pop, uint32_t record_words, uint
     }
 }
 
-// Bit (r, c) of the warp's 32 x 32 bit matrix (lane r's bit c) moves to (c, r).
-__device__ __forceinline__ uint32_t transpose32(uint32_t x, uint32_t lane)
-{
-    uint32_t y = __shfl_xor_sync(0xffffffffu, x, 16);
-    x = __byte_perm(x, y, (lane & 16u) ? 0x3276u : 0x5410u);
-    y = __shfl_xor_sync(0xffffffffu, x, 8);
-    x = __byte_perm(x, y, (lane & 8u) ? 0x3715u : 0x6240u);
-#pragma unroll
-    for (uint32_t j = 4u; j > 0u; j >>= 1) {
-        const uint32_t low = j == 4u ? 0x0F0F0F0Fu : j == 2u ? 0x33333333u : 0x55555555u;
-        const uint32_t keep = (lane & j) ? ~low : low;
-        y = __shfl_xor_sync(0xffffffffu, x, static_cast<int>(j));
-        y = __funnelshift_l(y, y, (lane & j) ? 32u - j : j);
-        x = (x & keep) | (y & ~keep);
-    }
-    return x;
-}
-
 // Block (x, y): rows i in [32 y, 32 y + 32), columns j in [64 x, 64 x + 64), pairs i < j.
 __global__ void __launch_bounds__(kMixThreads)
 mixed_pair_kernel(uint32_t n, uint32_t sites, uint32_t words, uint32_t bits, uint32_t K,
@@ -637,13 +502,14 @@ mixed_pair_kernel(uint32_t n, uint32_t sites, uint32_t words, uint32_t bits, uin
     const uint32_t i0 = blockIdx.y * kMixRows, j0 = blockIdx.x * kMixCols;
     if (j0 + kMixCols <= i0 + 1u) return;  // whole tile on or below the diagonal
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+    const Transpose32 transpose(lane);
     auto first_of = [&](uint32_t g) { return g == 0u ? i0 : j0 + 32u * (g - 1u); };
     wait_previous_grid();
     for (uint32_t t = warp; t < 3u * words; t += kMixThreads / 32u) {
         const uint32_t g = t / words, w = t - g * words;
         const uint32_t a = first_of(g) + lane;
         const uint32_t v = a < n ? __ldg(&surf[static_cast<size_t>(a) * words + w]) : 0u;
-        plane[g][32u * w + lane] = transpose32(v, lane);
+        plane[g][32u * w + lane] = transpose(v);
     }
     if (threadIdx.x < 96u) {
         const uint32_t g = threadIdx.x >> 5, a = first_of(g) + lane;
@@ -670,7 +536,7 @@ mixed_pair_kernel(uint32_t n, uint32_t sites, uint32_t words, uint32_t bits, uin
                         differ |= plane[ga][q] ^ (0u - ((plane[gb][q] >> bl) & 1u));
                 }
             }
-            const uint32_t x = transpose32(differ, lane);
+            const uint32_t x = transpose(differ);
             if (open && x != 0u) {
                 first = c0 + static_cast<uint32_t>(__ffs(static_cast<int>(x))) - 1u;
                 open = false;
@@ -747,7 +613,7 @@ size_t mrca_scratch_bytes(const ga_run *run, uint32_t n)
         MixedLayout l;
         return carve_mixed(nullptr, S, run->cfg.differentia_bits, n, l);
     }
-    return sync_scratch_bytes(S, n);
+    return sync_scratch_bytes(S, run->cfg.differentia_bits, n);
 }
 
 namespace {
@@ -784,15 +650,11 @@ cudaError_t launch_mrca(ga_run *run, const uint32_t *d_ids, uint32_t n, uint32_t
     if (run->cfg.mode != GA_SYNC) return launch_mrca_mixed(run, d_ids, n, d_lo, d_hi, scratch);
     const uint32_t S = run->cfg.surface_sites, b = run->cfg.differentia_bits;
     const uint32_t T = static_cast<uint32_t>(run->generation);
-    MrcaLayout l = carve(scratch, S);
-    uint32_t launches = 0;
-    const cudaError_t e = launch_sync_mrca(
-        reinterpret_cast<const uint32_t *>(run->pop[run->cur]), run->record_bytes / 4u,
-        run->n_agents, d_ids, n, l, run->cfg.curation, run->log2_sites, S, b, T, d_lo, d_hi,
-        run->d_status, run->stream, launches);
-    run->launches += launches;
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    const cudaError_t e =
+        launch_sync_mrca(run->pop[run->cur], run->record_bytes, run->n_agents, d_ids, n, scratch, run->cfg.curation,
+                         run->log2_sites, S, b, T, d_lo, d_hi, run->d_status, run->stream);
+    if (e == cudaSuccess) run->launches += 2;
+    return e;
 }
 
 }  // namespace ga
@@ -808,8 +670,8 @@ cudaError_t launch_mrca(ga_run *run, const uint32_t *d_ids, uint32_t n, uint32_t
 // up with cudaGetSymbolAddress, with the caller's device current, and passes it to the
 // kernels (a lookup per call stays right after a device reset reloads the module, which a
 // cached address would not).  Every call on a device reuses the same array: the status word
-// is cleared at the start of each call, the rank table and strings are fully rewritten
-// before they are read.
+// is cleared at the start of each call, the table and strings are fully rewritten before
+// they are read.
 // ---------------------------------------------------------------------------------------
 namespace ga {
 namespace {
@@ -817,10 +679,8 @@ namespace {
 constexpr uint32_t kFixedMaxSample = 4096;    // largest n accepted
 constexpr uint32_t kFixedMaxSites = 256;      // S * b <= 256 bits
 constexpr size_t kFixedStatusBytes = 256;     // device status word, padded
-// status, then the layout carve() gives the per-call scratch, sized for S = 256, n = 4096:
-// 256 + 2 x 1,024 + 256 + 4,096 x 32 = 133,632 bytes
-constexpr size_t kFixedScratchBytes = kFixedStatusBytes + 2 * 1024 + 256 +
-                                      static_cast<size_t>(kFixedMaxSample) * kPackWords * 4;
+// status, then the scratch of a call with n = 4096 and S = 256: 256 + 2,304 + 4,096 x 32 bytes
+constexpr size_t kFixedScratchBytes = kFixedStatusBytes + kTableBytes + static_cast<size_t>(kFixedMaxSample) * 32u;
 
 static __device__ __align__(256) unsigned char g_mrca_fixed_scratch[kFixedScratchBytes];
 
@@ -843,9 +703,6 @@ extern "C" int ga_mrca_bounds_noalloc(const void *d_records, uint32_t record_byt
     const uint32_t words = (S * b + 31u) / 32u;
     if (record_bytes != (8u + 4u * words + 15u) / 16u * 16u || n_agents == 0u) return GA_EINVAL;
     if (reinterpret_cast<uintptr_t>(d_records) % 16u != 0u) return GA_EINVAL;
-    static_assert(kFixedStatusBytes + 2 * 1024 + 256 + kFixedMaxSample * kPackWords * 4 <=
-                      kFixedScratchBytes, "fixed scratch too small for its largest call");
-
     // an error left pending by earlier, unrelated work on this thread is not this call's
     cudaGetLastError();
     void *base = nullptr;
@@ -855,15 +712,12 @@ extern "C" int ga_mrca_bounds_noalloc(const void *d_records, uint32_t record_byt
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int *status = static_cast<int *>(base);
-    MrcaLayout l = carve(static_cast<uint8_t *>(base) + kFixedStatusBytes, S);
     uint32_t log2_sites = 0;
     while ((1u << log2_sites) < S) ++log2_sites;
 
     if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return GA_ECUDA;
-    uint32_t launches = 0;
-    if (launch_sync_mrca(static_cast<const uint32_t *>(d_records), record_bytes / 4u, n_agents,
-                         d_agent_ids, n, l, curation, log2_sites, S, b, generation, d_lo, d_hi,
-                         status, st, launches) != cudaSuccess)
+    if (launch_sync_mrca(d_records, record_bytes, n_agents, d_agent_ids, n,
+                         static_cast<uint8_t *>(base) + kFixedStatusBytes, curation, log2_sites, S, b, generation, d_lo, d_hi, status, st) != cudaSuccess)
         return GA_ECUDA;
     int device_status = GA_OK;
     if (cudaMemcpyAsync(&device_status, status, sizeof(int), cudaMemcpyDeviceToHost, st) !=

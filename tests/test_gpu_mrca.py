@@ -56,6 +56,24 @@ def test_narrow_strings(S, b, policy, n_ids):
     assert np.array_equal(hi, ehi)
 
 
+@pytest.mark.parametrize("n_ids", [2, 3, 33, 257])
+@pytest.mark.parametrize("S,b,policy", [
+    (16, 2, "TILTED"), (64, 2, "HYBRID"), (128, 1, "STEADY"), (16, 8, "STEADY"), (32, 8, "HYBRID"),
+])
+def test_string_widths_and_small_samples(S, b, policy, n_ids):
+    """Strings of one, four and eight words (records of 16, 32 and 48 bytes) and samples around a
+    warp and a pack block, at a counter past every surface's size and one below it."""
+    from paper_2405_03605_gb300 import workloads
+    shape = RunShape(rows=3, cols=4, surface_sites=S, differentia_bits=b,
+                     curation=getattr(workloads, policy), seed=S * b)
+    for gens in (S // 2, 400):
+        g, o, ids = both(shape, gens, n_ids, seed=n_ids)
+        lo, hi = g.mrca_bounds(ids)
+        elo, ehi = o.mrca_bounds(ids)
+        assert np.array_equal(lo, elo)
+        assert np.array_equal(hi, ehi)
+
+
 def test_device_entry_point_matches_host():
     import torch
     shape = RunShape(rows=8, cols=8, seed=9)
