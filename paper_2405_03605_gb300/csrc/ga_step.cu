@@ -26,12 +26,13 @@ __global__ void __launch_bounds__(kStepThreads) island_step_kernel(const StepArg
 // equal the generation, islands of 16, 32 or 64 agents, any tournament size, both genome
 // models; TS = 0 reads the tournament size from the run.
 // Resident blocks per SM asked of the compiler: 8 (32 registers) below 64 agents; the two
-// agents per lane of 64-agent islands need 40 registers (6 blocks).
-template <int N>
-constexpr int units_min_blocks() { return N >= 64 ? 6 : 8; }
+// agents per lane of 64-agent islands need 40 registers (6 blocks).  The float model, 4: its
+// deviates need 64 (50 generations of 16.8M agents: 7,433 us; 7,638 with 5 blocks, 7,865 with 3).
+template <int N, int MODEL>
+constexpr int units_min_blocks() { return MODEL == 1 ? 4 : N >= 64 ? 6 : 8; }
 
 template <int N, int TS, int MODEL>
-__global__ void __launch_bounds__(kStepThreads, units_min_blocks<N>()) island_units_kernel(const StepArgs a)
+__global__ void __launch_bounds__(kStepThreads, (units_min_blocks<N, MODEL>())) island_units_kernel(const StepArgs a)
 {
     wait_previous_grid();
     step_units<N, TS, units_per_block<N>(), MODEL>(a.r, a.rk, blockIdx.x);

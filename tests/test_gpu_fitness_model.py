@@ -56,3 +56,23 @@ def test_fitness_runs_step_solo_inside_a_batch():
         assert_same(r.snapshot(), o.snapshot(), s.island_size)
     batch.close()
 
+
+
+@pytest.mark.parametrize("p_del,p_ben", [(0.0, 0.0), (0.33, 0.003), (0.5, 0.5), (1.0, 0.0)])
+@pytest.mark.parametrize("N,n,rows,cols,every", [
+    (32, 5, 5, 13, 1), (32, 3, 5, 13, 1), (32, 5, 1, 1, 1), (16, 5, 3, 11, 1), (16, 8, 3, 45, 2),
+    (64, 5, 5, 13, 1), (64, 2, 3, 5, 3),
+])
+def test_streamed_mutation_queue(N, n, rows, cols, every, p_del, p_ben):
+    """The streamed kernel works through queues of mutating births: none, a third, every birth of
+    a block's units, last units and islands missing, both tournament forms, every island size,
+    several generations to a launch."""
+    shape = RunShape(rows=rows, cols=cols, island_size=N, tournament_size=n, p_ben=p_ben, p_del=p_del,
+                     model=MODEL_FITNESS, effect_scale=0.5, migrate_every=every, seed=41 + N + n, run_id=rows)
+    g = gpu_run(shape)
+    g.resident_policy(1)  # GA_RESIDENT_OFF
+    g.step(40)
+    g.sync()
+    o = oracle_for(shape)
+    o.step(40)
+    assert_same(g.snapshot(), o.snapshot(), N)
