@@ -400,12 +400,11 @@ cudaError_t launch_sync_mrca(const void *pop, uint32_t record_bytes, uint32_t n_
 //                      agent), so lane l looks up the mismatches of all 32 agents at b's l-th
 //                      rank in one word, and a 32 x 32 bit transpose hands every lane its own
 //                      agent's mismatches in b's rank order: the first set bit is the answer.
-// Issue-bound: 239 warp-instructions per 32 pairs at 75% issue, against 2,757 for one thread per
-// pair walking both agents' sites twice.  The whole call for 3,001 agents with 64 sites (4.5M
-// pairs, 36 MB of bounds): 50 us, 376 us before.
+// Issue-bound: some 200 warp-instructions per 32 pairs, against 2,757 for one thread per pair
+// walking both agents' sites twice.  The whole call for 3,001 agents with 64 sites (4.5M pairs, 36
+// MB of bounds): 47 us, 376 us before; 2,816 agents with 256 sites 122 us, 1,371 before.
 // ---------------------------------------------------------------------------------------
 constexpr uint32_t kMixRows = 32, kMixCols = 64;
-constexpr uint32_t kMixThreads = 256;
 constexpr uint32_t kMixPad = kMixCols + 1;  // staged bounds: row stride without bank conflicts
 
 struct MixedLayout {
@@ -484,8 +483,11 @@ mixed_table_kernel(const uint32_t *__restrict__ pop, uint32_t record_words, uint
     }
 }
 
-// Block (x, y): rows i in [32 y, 32 y + 32), columns j in [64 x, 64 x + 64), pairs i < j.
-__global__ void __launch_bounds__(kMixThreads)
+// Block (x, y): rows i in [32 y, 32 y + 32), columns j in [64 x, 64 x + 64), pairs i < j.  THREADS:
+// 256, or 1,024 where there are fewer tiles than two for each SM (a tile's 128 steps then take a
+// quarter of the time: 249 agents 12.6 us, 20 with 256).  BIT: one-bit differentiae.
+template <uint32_t THREADS, bool BIT>
+__global__ void __launch_bounds__(THREADS)
 mixed_pair_kernel(uint32_t n, uint32_t sites, uint32_t words, uint32_t bits, uint32_t K,
                   const uint32_t *__restrict__ cnt, const uint32_t *__restrict__ held,
                   const uint32_t *__restrict__ surf, const uint32_t *__restrict__ ranks,
@@ -505,7 +507,7 @@ mixed_pair_kernel(uint32_t n, uint32_t sites, uint32_t words, uint32_t bits, uin
     const Transpose32 transpose(lane);
     auto first_of = [&](uint32_t g) { return g == 0u ? i0 : j0 + 32u * (g - 1u); };
     wait_previous_grid();
-    for (uint32_t t = warp; t < 3u * words; t += kMixThreads / 32u) {
+    for (uint32_t t = warp; t < 3u * words; t += THREADS / 32u) {
         const uint32_t g = t / words, w = t - g * words;
         const uint32_t a = first_of(g) + lane;
         const uint32_t v = a < n ? __ldg(&surf[static_cast<size_t>(a) * words + w]) : 0u;
@@ -518,74 +520,105 @@ mixed_pair_kernel(uint32_t n, uint32_t sites, uint32_t words, uint32_t bits, uin
     }
     __syncthreads();
 
-    // The pairs of agent b (lane bl of group gb, index nb in the sample) with the agents of
-    // group ga (one per lane, counters at most b's where `active`): bounds of each lane's pair.
-    auto pairs_of = [&](uint32_t gb, uint32_t bl, uint32_t nb, uint32_t ga, uint32_t Ta, bool active,
-                        uint32_t &l, uint32_t &h) {
+    // The pairs of agent b (lane bl of group gb, index nb in the sample) with the agents of NG
+    // groups from ga on (one per lane each, counters at most b's where `active`): bounds of each
+    // lane's pairs.  site0: b's site at rank index `lane`, read a step ahead.
+    auto pairs_of = [&](auto groups, uint32_t gb, uint32_t bl, uint32_t nb, uint32_t ga, uint32_t site0,
+                        const uint32_t *Ta, const bool *active, uint32_t *l, uint32_t *h) {
+        constexpr int NG = decltype(groups)::value;
         const uint32_t m = held_s[gb][bl];
         const uint32_t *rk = ranks + static_cast<size_t>(nb) * sites;
         const uint8_t *od = order + static_cast<size_t>(nb) * sites;
-        uint32_t first = kNone;  // first index in b's rank order whose differentiae differ
-        bool open = active;
+        uint32_t first[NG];  // first index in b's rank order whose differentiae differ
+        bool open[NG], any = false;
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            first[g] = kNone;
+            open[g] = active[g];
+        }
         for (uint32_t c0 = 0; c0 < m; c0 += 32u) {
-            uint32_t differ = 0;  // bit a: agent a differs from b at b's (c0 + lane)-th rank
+            uint32_t differ[NG];  // bit a: agent a differs from b at b's (c0 + lane)-th rank
+#pragma unroll
+            for (int g = 0; g < NG; ++g) differ[g] = 0u;
             if (c0 + lane < m) {
-                const uint32_t q0 = __ldg(&od[c0 + lane]) * bits;
+                const uint32_t q0 = (c0 == 0u ? site0 : __ldg(&od[c0 + lane])) * (BIT ? 1u : bits);
                 if (in_bounds(q0 + bits <= 32u * words, status)) {
-                    for (uint32_t q = q0; q < q0 + bits; ++q)
-                        differ |= plane[ga][q] ^ (0u - ((plane[gb][q] >> bl) & 1u));
+                    for (uint32_t q = q0; q < q0 + (BIT ? 1u : bits); ++q) {
+                        const uint32_t mine = 0u - ((plane[gb][q] >> bl) & 1u);
+#pragma unroll
+                        for (int g = 0; g < NG; ++g) differ[g] |= plane[ga + g][q] ^ mine;
+                    }
                 }
             }
-            const uint32_t x = transpose(differ);
-            if (open && x != 0u) {
-                first = c0 + static_cast<uint32_t>(__ffs(static_cast<int>(x))) - 1u;
-                open = false;
+            any = false;
+#pragma unroll
+            for (int g = 0; g < NG; ++g) {
+                const uint32_t x = transpose(differ[g]);
+                if (open[g] && x != 0u) {
+                    first[g] = c0 + static_cast<uint32_t>(__ffs(static_cast<int>(x))) - 1u;
+                    open[g] = false;
+                }
+                any = any || open[g];
             }
-            if (!__any_sync(0xffffffffu, open)) break;
+            if (!__any_sync(0xffffffffu, any)) break;
         }
-        if (!active) return;
-        // a mismatch at a rank not below Ta lies past the common prefix
-        uint32_t end = first;
-        h = Ta;
-        const uint32_t fr = first != kNone ? __ldg(&rk[first]) : kNone;
-        if (fr < Ta) {
-            h = fr;
-        } else {  // no common rank differs: the prefix ends at the first rank >= Ta
-            uint32_t below = 0, above = m;
-            while (below < above) {
-                const uint32_t mid = (below + above) >> 1;
-                if (__ldg(&rk[mid]) < Ta) below = mid + 1u;
-                else above = mid;
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            if (!active[g]) continue;
+            // a mismatch at a rank not below Ta lies past the common prefix
+            const uint32_t fr = first[g] != kNone ? __ldg(&rk[first[g]]) : kNone;
+            const uint32_t fl = first[g] != kNone && first[g] >= K ? __ldg(&rk[first[g] - K]) + 1u : 0u;
+            h[g] = fr;
+            l[g] = fl;
+            if (fr >= Ta[g]) {  // no common rank differs: the prefix ends at the first rank >= Ta
+                uint32_t below = 0, above = m;
+                while (below < above) {
+                    const uint32_t mid = (below + above) >> 1;
+                    if (__ldg(&rk[mid]) < Ta[g]) below = mid + 1u;
+                    else above = mid;
+                }
+                h[g] = Ta[g];
+                l[g] = below >= K ? __ldg(&rk[below - K]) + 1u : 0u;
             }
-            end = below;
         }
-        l = end >= K ? __ldg(&rk[end - K]) + 1u : 0u;
+    };
+    // the site at rank index `lane` of sampled agent a (0 where there is none)
+    auto first_site = [&](uint32_t a) {
+        return a < n && lane < sites ? static_cast<uint32_t>(__ldg(&order[static_cast<size_t>(a) * sites + lane])) : 0u;
     };
 
     // pairs whose row agent holds the larger counter (or the same): b = row, lanes = columns
-    for (uint32_t r = warp; r < kMixRows; r += kMixThreads / 32u) {
-        const uint32_t i = i0 + r, Tb = count[0][r];
+    uint32_t ahead = first_site(i0 + warp);
+    for (uint32_t r = warp; r < kMixRows; r += THREADS / 32u) {
+        const uint32_t i = i0 + r, Tb = count[0][r], site0 = ahead;
+        if (r + THREADS / 32u < kMixRows) ahead = first_site(i + THREADS / 32u);
+        uint32_t Ta[2], l[2], h[2];
+        bool active[2];
 #pragma unroll
-        for (uint32_t g = 1; g <= 2u; ++g) {
-            const uint32_t j = first_of(g) + lane, Ta = count[g][lane];
-            const bool active = i < j && j < n && Ta <= Tb;
-            if (!__any_sync(0xffffffffu, active)) continue;
-            uint32_t l = 0, h = 0;
-            pairs_of(0u, r, i, g, Ta, active, l, h);
-            if (active) {
-                s_lo[r][32u * (g - 1u) + lane] = l;
-                s_hi[r][32u * (g - 1u) + lane] = h;
-            }
+        for (uint32_t g = 0; g < 2u; ++g) {
+            const uint32_t j = j0 + 32u * g + lane;
+            Ta[g] = count[1u + g][lane];
+            active[g] = i < j && j < n && Ta[g] <= Tb;
         }
+        if (!__any_sync(0xffffffffu, active[0] || active[1])) continue;
+        pairs_of(std::integral_constant<int, 2>(), 0u, r, i, 1u, site0, Ta, active, l, h);
+#pragma unroll
+        for (uint32_t g = 0; g < 2u; ++g)
+            if (active[g]) {
+                s_lo[r][32u * g + lane] = l[g];
+                s_hi[r][32u * g + lane] = h[g];
+            }
     }
     // pairs whose column agent holds the larger counter: b = column, lanes = rows
-    for (uint32_t c = warp; c < kMixCols; c += kMixThreads / 32u) {
-        const uint32_t g = 1u + (c >> 5), bl = c & 31u;
+    ahead = first_site(j0 + warp);
+    for (uint32_t c = warp; c < kMixCols; c += THREADS / 32u) {
+        const uint32_t g = 1u + (c >> 5), bl = c & 31u, site0 = ahead;
         const uint32_t i = i0 + lane, j = j0 + c, Ta = count[0][lane];
+        if (c + THREADS / 32u < kMixCols) ahead = first_site(j + THREADS / 32u);
         const bool active = i < j && j < n && Ta < count[g][bl];
         if (!__any_sync(0xffffffffu, active)) continue;
         uint32_t l = 0, h = 0;
-        pairs_of(g, bl, j, 0u, Ta, active, l, h);
+        pairs_of(std::integral_constant<int, 1>(), g, bl, j, 0u, site0, &Ta, &active, &l, &h);
         if (active) {
             s_lo[lane][c] = l;
             s_hi[lane][c] = h;
@@ -593,7 +626,7 @@ mixed_pair_kernel(uint32_t n, uint32_t sites, uint32_t words, uint32_t bits, uin
     }
     __syncthreads();
     // the tile's bounds, row by row in output order
-    for (uint32_t t = threadIdx.x; t < kMixRows * kMixCols; t += kMixThreads) {
+    for (uint32_t t = threadIdx.x; t < kMixRows * kMixCols; t += THREADS) {
         const uint32_t r = t / kMixCols, c = t % kMixCols;
         const uint32_t i = i0 + r, j = j0 + c;
         if (i < j && j < n) {
@@ -634,7 +667,10 @@ cudaError_t launch_mrca_mixed(ga_run *run, const uint32_t *d_ids, uint32_t n, ui
     if (e != cudaSuccess) return e;
     run->launches += 1;
     const dim3 grid((n + kMixCols - 1u) / kMixCols, (n + kMixRows - 1u) / kMixRows);
-    e = launch_dependent(mixed_pair_kernel, grid, kMixThreads, run->stream, n, S, words, b, margin(b),
+    const bool few = grid.x * grid.y / 2u < 2u * 152u;
+    const auto kernel = few ? (b == 1u ? mixed_pair_kernel<1024, true> : mixed_pair_kernel<1024, false>)
+                            : (b == 1u ? mixed_pair_kernel<256, true> : mixed_pair_kernel<256, false>);
+    e = launch_dependent(kernel, grid, few ? 1024u : 256u, run->stream, n, S, words, b, margin(b),
                          static_cast<const uint32_t *>(l.cnt), static_cast<const uint32_t *>(l.held),
                          static_cast<const uint32_t *>(l.surf), static_cast<const uint32_t *>(l.ranks),
                          static_cast<const uint8_t *>(l.order), d_lo, d_hi, run->d_status);
