@@ -155,6 +155,18 @@ __device__ __forceinline__ void island_draws(uint4 (&w)[Shape<N>::A], const Slot
     }
 }
 
+// Shared memory of a warp for islands of more than 32 agents: a lookup by slot is one load there
+// (at most two wavefronts for 64 agents), where shuffles read every register a lane holds and
+// choose.  traits: two sets of N used in turn by generation; surfaces: SW / 2 arrays of N (islands
+// of 128 only; for 64 the shuffles of whole surfaces take fewer wavefronts).  4.2M agents of 48
+// bytes in islands of 64, migration every 16 generations: 23.2 -> 20.7 us per generation with the
+// traits there; islands of 128 every generation, 4.2M agents of 16 bytes 37.5 -> 27.5, of 48 bytes
+// 102.8 -> 76.8.
+struct Lookup {
+    int *traits = nullptr;
+    uint2 *surfaces = nullptr;
+};
+
 // Evaluation, tournament, copy, mutation and hstrat deposit of one generation, in place.
 // Closed-form curation site, called only for agents whose counter differs from the
 // generation (never in synchronous runs); kept out of line so the common path stays a load.
@@ -180,10 +192,26 @@ __device__ __forceinline__ void reproduce(uint32_t (&rec)[Shape<N>::A][2 + SW],
                                           const RoundKeys &rk, uint32_t island, uint32_t seg_lane,
                                           unsigned mask, uint32_t g, int gen_site,
                                           uint2 dmask = make_uint2(0u, 0u),
-                                          const float *amount = nullptr, const bool *mutates = nullptr)
+                                          const float *amount = nullptr, const bool *mutates = nullptr,
+                                          const Lookup lookup = {})
 {
     constexpr int A = Shape<N>::A, SEG = Shape<N>::SEG, LOGN = Shape<N>::LOGN;
     constexpr int LW = 2 + SW;
+    // islands of more than 32: traits, and of 128 surfaces, through shared memory
+    const bool shared = N > 32 && lookup.traits != nullptr;
+    if constexpr (N > 32) {
+        if (shared) {
+#pragma unroll
+            for (int ag = 0; ag < A; ++ag) {
+                lookup.traits[seg_lane + 32u * ag] = static_cast<int>(rec[ag][0]);
+                if constexpr (N > 64)
+#pragma unroll
+                    for (int k = 0; k < SW / 2; ++k)
+                        lookup.surfaces[k * N + seg_lane + 32u * ag] = make_uint2(rec[ag][2 + 2 * k], rec[ag][3 + 2 * k]);
+            }
+            __syncwarp();
+        }
+    }
     // tournament: best of n draws with replacement, earliest wins ties; draw i's slot is byte
     // (i mod 4) of B0 / B1 scaled to N, i.e. that byte's top log2 N bits
     int trait[A];
@@ -201,7 +229,7 @@ __device__ __forceinline__ void reproduce(uint32_t (&rec)[Shape<N>::A][2 + SW],
                 const uint32_t word = i < 4 ? w[ag].x : w[ag].y;
                 uint32_t sel = word >> (8 * (i & 3) + 8 - LOGN);
                 if constexpr (N > 32) sel &= N - 1u;
-                const int t = candidate_trait<N, A, SEG>(mask, trait, sel);
+                const int t = shared ? lookup.traits[sel] : candidate_trait<N, A, SEG>(mask, trait, sel);
                 bool better;
                 if constexpr (MODEL == 1) better = __int_as_float(t) > __int_as_float(best_trait);
                 else better = t > best_trait;
@@ -220,7 +248,7 @@ __device__ __forceinline__ void reproduce(uint32_t (&rec)[Shape<N>::A][2 + SW],
                 const uint32_t word = i < 4 ? w[ag].x : w[ag].y;
                 uint32_t sel = word >> (8 * (i & 3) + 8 - LOGN);
                 if constexpr (N > 32) sel &= N - 1u;
-                const int t = candidate_trait<N, A, SEG>(mask, trait, sel);
+                const int t = shared ? lookup.traits[sel] : candidate_trait<N, A, SEG>(mask, trait, sel);
                 bool better;
                 if constexpr (MODEL == 1) better = __int_as_float(t) >= __int_as_float(best_trait);
                 else better = t >= best_trait;
@@ -261,6 +289,11 @@ __device__ __forceinline__ void reproduce(uint32_t (&rec)[Shape<N>::A][2 + SW],
                 child[ag][1] = g;
                 continue;
             }
+            if (N > 64 && shared && k >= 2) {
+                const uint2 v = lookup.surfaces[(k - 2) / 2 * N + win[ag]];
+                child[ag][k] = (k & 1) ? v.y : v.x;
+                continue;
+            }
             if constexpr (N <= 32) {
                 child[ag][k] = __shfl_sync(mask, rec[0][k], static_cast<int>(win[ag]), SEG);
             } else {
@@ -274,6 +307,8 @@ __device__ __forceinline__ void reproduce(uint32_t (&rec)[Shape<N>::A][2 + SW],
             }
         }
     }
+
+    if (N > 64 && shared) __syncwarp();  // the surfaces have been read
 
     // mutation and hstrat deposit
 #pragma unroll
@@ -309,6 +344,8 @@ __device__ __forceinline__ void reproduce(uint32_t (&rec)[Shape<N>::A][2 + SW],
             const uint32_t rep = (w[ag].w & p.dif_mask) * p.dif_rep;
             child[ag][2] = (child[ag][2] & ~dmask.x) | (rep & dmask.x);
             child[ag][3] = (child[ag][3] & ~dmask.y) | (rep & dmask.y);
+        } else if constexpr (CF == 0 && SW > 2) {
+            // below, for all the lane's agents at once
         } else if (site >= 0 && in_bounds(static_cast<uint32_t>(site) < p.sites &&
                                               site * p.bits < 32u * SW,
                                           p.status)) {
@@ -323,6 +360,32 @@ __device__ __forceinline__ void reproduce(uint32_t (&rec)[Shape<N>::A][2 + SW],
         child[ag][1] = c + 1u;
 #pragma unroll
         for (int k = 0; k < LW; ++k) rec[ag][k] = child[ag][k];
+    }
+    if constexpr (CF == 0 && SW > 2) {
+        // uniform counters: one site for every agent, so one jump to its surface word (a test and a
+        // select for each of eight words before: 4.2M agents in islands of 64, migration every 16
+        // generations, 24.3 -> 23.2 us per generation)
+        if (gen_site >= 0 && in_bounds(static_cast<uint32_t>(gen_site) < p.sites && gen_site * p.bits < 32u * SW, p.status)) {
+            const uint32_t pos = static_cast<uint32_t>(gen_site) * p.bits, sh = pos & 31u;
+            const uint32_t m = p.dif_mask << sh;
+            auto put = [&](auto word) {
+                constexpr int k = 2 + decltype(word)::value;
+                if constexpr (k < LW) {
+#pragma unroll
+                    for (int ag = 0; ag < A; ++ag) rec[ag][k] = (rec[ag][k] & ~m) | ((w[ag].w << sh) & m);
+                }
+            };
+            switch (pos >> 5) {
+            case 0: put(std::integral_constant<int, 0>()); break;
+            case 1: put(std::integral_constant<int, 1>()); break;
+            case 2: put(std::integral_constant<int, 2>()); break;
+            case 3: put(std::integral_constant<int, 3>()); break;
+            case 4: put(std::integral_constant<int, 4>()); break;
+            case 5: put(std::integral_constant<int, 5>()); break;
+            case 6: put(std::integral_constant<int, 6>()); break;
+            default: put(std::integral_constant<int, 7>()); break;
+            }
+        }
     }
 }
 
@@ -486,13 +549,24 @@ __device__ __forceinline__ void step_block(const RunParams &p, const RoundKeys &
             }
         }
     }
-    reproduce<N, SW, TS, MODEL, CF>(rec, w, p, rk, island, seg_lane, mask, p.g0, gen_site_at(p, 0u));
+    constexpr bool kShared = N > 32, kSurfaces = N > 64;
+    __shared__ int s_trait[kShared ? WARPS : 1][kShared ? 2 : 1][kShared ? N : 1];
+    __shared__ uint2 s_surf[kSurfaces ? WARPS : 1][kSurfaces ? SW / 2 * N : 1];
+    const uint32_t warp = threadIdx.x >> 5;
+    auto lookup = [&](uint32_t it) {
+        Lookup l;
+        if constexpr (kShared) l.traits = s_trait[warp][it & 1u];
+        if constexpr (kSurfaces) l.surfaces = s_surf[warp];
+        return l;
+    };
+    reproduce<N, SW, TS, MODEL, CF>(rec, w, p, rk, island, seg_lane, mask, p.g0, gen_site_at(p, 0u),
+                                    make_uint2(0u, 0u), nullptr, nullptr, lookup(0u));
 
     // generations g0 + 1 .. g0 + n - 1: no migration, the island stays in registers
     for (uint32_t it = 1; it < p.n_gens; ++it) {
         birth_draws<N>(w, p, rk, p.g0 + it, island, seg_lane);
         reproduce<N, SW, TS, MODEL, CF>(rec, w, p, rk, island, seg_lane, mask, p.g0 + it,
-                                        gen_site_at(p, it));
+                                        gen_site_at(p, it), make_uint2(0u, 0u), nullptr, nullptr, lookup(it));
     }
 
 #pragma unroll
@@ -621,6 +695,18 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
     }
     __syncthreads();
 
+    // traits through shared memory from a launch's second generation on (4.2M agents in islands of
+    // 64, migration every 16 generations: 19.9 -> 17.6 us per generation; the first alone is 4%
+    // slower with it)
+    constexpr bool kShared = N > 32;
+    __shared__ int s_trait[kShared ? WARPS : 1][kShared ? 2 : 1][kShared ? N : 1];
+    uint32_t turn = 0;
+    auto lookup = [&]() {  // the next generation's set
+        Lookup l;
+        if constexpr (kShared) l.traits = s_trait[warp][turn++ & 1u];
+        return l;
+    };
+
     const uint2 dmask = gen_mask_at(p, 0u);
     const SlotDraws<N> sd = slot_draws<N>(p, rk, p.g0, seg_lane);
     // UNROLL: fully unrolled over the block's units, so the double-buffer index, the
@@ -726,7 +812,7 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
                 for (uint32_t it = 1; it < p.n_gens; ++it) {
                     birth_draws<N>(w, p, rk, p.g0 + it, island, seg_lane);
                     reproduce<N, SW, TS, 1, 0, 1>(rec, w, p, rk, island, seg_lane, mask, p.g0 + it, 0,
-                                                  gen_mask_at(p, it));
+                                                  gen_mask_at(p, it), nullptr, nullptr, lookup());
                 }
                 uint4 *dst = p.dst + static_cast<size_t>(first) * N + lane;
 #pragma unroll
@@ -778,7 +864,7 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
         for (uint32_t it = 1; it < p.n_gens; ++it) {
             birth_draws<N>(w, p, rk, p.g0 + it, island, seg_lane);
             reproduce<N, SW, TS, MODEL, 0, 1>(rec, w, p, rk, island, seg_lane, mask, p.g0 + it, 0,
-                                              gen_mask_at(p, it));
+                                              gen_mask_at(p, it), nullptr, nullptr, lookup());
         }
         uint4 *dst = p.dst + static_cast<size_t>(first) * N + lane;
 #pragma unroll

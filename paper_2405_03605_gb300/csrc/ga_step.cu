@@ -115,42 +115,36 @@ StepKernel pick_fitness(uint32_t surface_words, uint32_t tsize)
 }
 
 // Kernels without the closed-form curation path, for launches whose counters all equal the
-// generation, tournament size 5 (the paper's, Sec. 3): 16-byte trait records for every island
-// size, 32- and 48-byte trait records and the float-fitness model for islands of 16, 32 and 64.
-template <int N>
-StepKernel pick_uniform_wide(uint32_t surface_words)
+// generation: 16-byte trait records of the island sizes that island_units_kernel does not take, and
+// 32- and 48-byte trait records of islands of 16 to 128.
+template <int N, int SW>
+StepKernel uniform_ts(uint32_t tsize)
 {
-    if (surface_words <= 6) return island_step_kernel<N, 6, 5, 0, 0>;
-    if (surface_words <= 8) return island_step_kernel<N, 8, 5, 0, 0>;
-    return nullptr;
+    return tsize == 5u ? island_step_kernel<N, SW, 5, 0, 0> : island_step_kernel<N, SW, 0, 0, 0>;
 }
 
-StepKernel pick_uniform(uint32_t island_size, uint32_t surface_words, uint32_t model)
+template <int N>
+StepKernel uniform_wide(uint32_t surface_words, uint32_t tsize)
 {
-    if (surface_words > 2) {
-        if (model != GA_MODEL_TRAIT) return nullptr;
+    return surface_words <= 6u ? uniform_ts<N, 6>(tsize) : uniform_ts<N, 8>(tsize);
+}
+
+StepKernel pick_uniform(uint32_t island_size, uint32_t surface_words, uint32_t tsize, uint32_t model)
+{
+    if (model != GA_MODEL_TRAIT) return nullptr;
+    if (surface_words > 2u) {
         switch (island_size) {
-        case 16: return pick_uniform_wide<16>(surface_words);
-        case 32: return pick_uniform_wide<32>(surface_words);
-        case 64: return pick_uniform_wide<64>(surface_words);
-        default: return nullptr;
-        }
-    }
-    if (model == GA_MODEL_FITNESS) {
-        switch (island_size) {
-        case 16: return island_step_kernel<16, 2, 5, 1, 0>;
-        case 32: return island_step_kernel<32, 2, 5, 1, 0>;
-        case 64: return island_step_kernel<64, 2, 5, 1, 0>;
+        case 16: return uniform_wide<16>(surface_words, tsize);
+        case 32: return uniform_wide<32>(surface_words, tsize);
+        case 64: return uniform_wide<64>(surface_words, tsize);
+        case 128: return uniform_wide<128>(surface_words, tsize);
         default: return nullptr;
         }
     }
     switch (island_size) {
-    case 4: return island_step_kernel<4, 2, 5, 0, 0>;
-    case 8: return island_step_kernel<8, 2, 5, 0, 0>;
-    case 16: return island_step_kernel<16, 2, 5, 0, 0>;
-    case 32: return island_step_kernel<32, 2, 5, 0, 0>;
-    case 64: return island_step_kernel<64, 2, 5, 0, 0>;
-    case 128: return island_step_kernel<128, 2, 5, 0, 0>;
+    case 4: return uniform_ts<4, 2>(tsize);
+    case 8: return uniform_ts<8, 2>(tsize);
+    case 128: return uniform_ts<128, 2>(tsize);
     default: return nullptr;
     }
 }
@@ -262,8 +256,7 @@ cudaError_t launch_counter_check(ga_run *run, uint32_t generation, int *d_flag)
 cudaError_t launch_island_step(ga_run *run, const void *src, void *dst, uint32_t g0,
                                uint32_t n_gens, bool migrate, cudaStream_t stream)
 {
-    const bool uniform = run->cfg.mode == GA_SYNC && run->counters_uniform &&
-                         run->cfg.tournament_size == 5;
+    const bool uniform = run->cfg.mode == GA_SYNC && run->counters_uniform;
     if (run->cfg.mode == GA_SYNC && run->counters_uniform && run->surface_words <= 2) {
         const uint32_t N = run->cfg.island_size, ts = run->cfg.tournament_size;
         const bool fit = run->cfg.model == GA_MODEL_FITNESS;
@@ -298,7 +291,8 @@ cudaError_t launch_island_step(ga_run *run, const void *src, void *dst, uint32_t
         }
     }
     StepKernel k =
-        uniform ? pick_uniform(run->cfg.island_size, run->surface_words, run->cfg.model) : nullptr;
+        uniform ? pick_uniform(run->cfg.island_size, run->surface_words, run->cfg.tournament_size, run->cfg.model)
+                : nullptr;
     if (!k)
         k = pick_kernel(run->cfg.island_size, run->surface_words, run->cfg.tournament_size,
                         run->cfg.model);

@@ -252,3 +252,55 @@ def test_benchmark_depth_10000_generations(shape):
     lo, hi = g.mrca_bounds(ids)
     elo, ehi = o.mrca_bounds(ids)
     assert np.array_equal(lo, elo) and np.array_equal(hi, ehi)
+
+
+@pytest.mark.parametrize("N,rows,cols,S,b,policy,every,tsize", [
+    (32, 5, 13, 256, 1, "STEADY", 1, 5), (32, 1, 1, 128, 1, "STEADY", 1, 3), (16, 3, 11, 256, 1, "HYBRID", 1, 8),
+    (64, 5, 13, 32, 8, "TILTED", 16, 5), (64, 3, 5, 128, 1, "STEADY", 7, 2), (32, 5, 9, 32, 8, "TILTED", 16, 5),
+    (16, 9, 15, 64, 2, "TILTED", 5, 5), (32, 4, 5, 32, 4, "HYBRID", 16, 4), (64, 2, 2, 64, 4, "STEADY", 0, 5),
+    (16, 33, 41, 32, 8, "STEADY", 16, 5), (32, 70, 90, 256, 1, "STEADY", 40, 5),
+])
+def test_streamed_wide_records(N, rows, cols, S, b, policy, every, tsize):
+    """The streamed kernel of 32- and 48-byte records: segments that end because the tag is full
+    (8-, 4- and 2-bit differentiae), because the launch ends, or never inside 256 generations; one
+    and several units to a block, missing last islands; padding that a load left nonzero."""
+    from paper_2405_03605_gb300 import workloads
+    shape = RunShape(rows=rows, cols=cols, island_size=N, tournament_size=tsize, surface_sites=S,
+                     differentia_bits=b, curation=getattr(workloads, policy), migrate_every=every,
+                     seed=91 + N + S, run_id=b, p_ben=0.05, p_del=0.05)
+    g, o = gpu_run(shape), oracle_for(shape)
+    g.resident_policy(1)  # GA_RESIDENT_OFF
+    for gens in (3, 150, 61):
+        g.step(gens)
+        g.sync()
+        o.step(gens)
+        assert_same(g.snapshot(), o.snapshot(), N)
+    if shape.record_bytes == 48:
+        rec = g.snapshot()
+        rec[:, 40:48] = 7
+        g.load(rec, 214)
+        g.step(2)
+        g.sync()
+        o.step(2)
+        assert_same(g.snapshot(), o.snapshot(), N)
+
+
+@pytest.mark.parametrize("N,rows,cols,S,b,policy,every,tsize,model", [
+    (128, 3, 7, 64, 1, "STEADY", 1, 5, 0), (128, 3, 3, 256, 1, "HYBRID", 4, 3, 0), (128, 1, 2, 128, 1, "STEADY", 16, 8, 0),
+    (128, 2, 5, 32, 8, "TILTED", 0, 5, 0), (64, 5, 7, 64, 1, "STEADY", 4, 5, 0), (64, 3, 5, 8, 8, "TILTED", 16, 2, 0),
+    (64, 5, 7, 64, 1, "STEADY", 3, 5, 1), (8, 7, 9, 64, 1, "STEADY", 4, 3, 0), (4, 5, 9, 64, 1, "STEADY", 2, 8, 0),
+])
+def test_streamed_lookups(N, rows, cols, S, b, policy, every, tsize, model):
+    """Islands of 64 and 128, whose traits (and surfaces, for 128) are looked up in shared memory, and
+    the kernels of uniform counters with a run-time tournament size: every record size, one and
+    several generations to a launch."""
+    from paper_2405_03605_gb300 import workloads
+    shape = RunShape(rows=rows, cols=cols, island_size=N, tournament_size=tsize, surface_sites=S,
+                     differentia_bits=b, curation=getattr(workloads, policy), migrate_every=every, model=model,
+                     seed=55 + N + S, run_id=every, p_ben=0.05, p_del=0.3 if model else 0.05)
+    g, o = gpu_run(shape), oracle_for(shape)
+    g.resident_policy(1)  # GA_RESIDENT_OFF
+    g.step(90)
+    g.sync()
+    o.step(90)
+    assert_same(g.snapshot(), o.snapshot(), N)
