@@ -551,7 +551,7 @@ __device__ __forceinline__ void step_block(const RunParams &p, const RoundKeys &
     }
     constexpr bool kShared = N > 32, kSurfaces = N > 64;
     __shared__ int s_trait[kShared ? WARPS : 1][kShared ? 2 : 1][kShared ? N : 1];
-    __shared__ uint2 s_surf[kSurfaces ? WARPS : 1][kSurfaces ? SW / 2 * N : 1];
+    __shared__ __align__(16) uint2 s_surf[kSurfaces ? WARPS : 1][kSurfaces ? SW / 2 * N : 1];
     const uint32_t warp = threadIdx.x >> 5;
     auto lookup = [&](uint32_t it) {
         Lookup l;
@@ -569,15 +569,42 @@ __device__ __forceinline__ void step_block(const RunParams &p, const RoundKeys &
                                         gen_site_at(p, it), make_uint2(0u, 0u), nullptr, nullptr, lookup(it));
     }
 
+    // 48-byte records go out through shared memory (space whose contents have been read: the
+    // island's part of the landing table, the warp's surfaces; else its own), 32 agents at a time
+    // and each store a full run of 128-byte lines: a lane's own three stores leave every line to
+    // be filled by three instructions.  256 sites, a migration per generation, us a generation:
+    // islands of 32: 2.78 against 3.16 for 65,536 agents, 16.7 against 18.6 for 1M, 66.1 against
+    // 69.9 for 4.2M; of 64: 62.1 against 68.1; of 128: 70.3 against 76.4.  With several
+    // generations to a launch the stores are few and the arithmetic bounds large runs, where the
+    // extra pass costs up to 4% (2 generations, islands of 32, 4.2M agents: 39.8 against 38.9;
+    // islands of 64: 37.3 against 39.4, even from 8 on); with at most 32,768 islands it still
+    // gains (262,144 agents, 4 generations: 2.15 against 2.26).  32-byte records, whose own stores
+    // fill whole sectors, are written directly: 53.6 us against 49.6 for 4.2M the other way.
+    constexpr bool kStaged = Q == 3, kOwn = kStaged && !kSlotTable && !kSurfaces;
+    __shared__ uint4 s_out[kOwn ? WARPS : 1][kOwn ? SEG * Q : 1];
+    uint4 *stage;
+    if constexpr (kSlotTable) stage = &s_in[local * N][0];
+    else if constexpr (kSurfaces) stage = reinterpret_cast<uint4 *>(s_surf[warp]);
+    else stage = s_out[kOwn ? warp : 0];
+    static_assert(!kStaged || !kSurfaces || SW / 2 * N * sizeof(uint2) >= SEG * Q * sizeof(uint4), "stage");
+    const bool staged = kStaged && (p.n_gens <= (N > 32 ? 4u : 1u) || p.n_islands <= 32768u);
 #pragma unroll
     for (int ag = 0; ag < A; ++ag) {
-        const size_t agent = static_cast<size_t>(island) * N + seg_lane + 32u * ag;
+        uint4 *out = p.dst + (static_cast<size_t>(island) * N + 32u * ag) * Q;  // this segment's records
+        if (staged) __syncwarp(mask);
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             uint32_t w4[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) w4[e] = (4 * q + e < LW) ? rec[ag][4 * q + e] : 0u;
-            p.dst[agent * Q + q] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+            const uint4 v = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+            if (staged) stage[seg_lane * Q + q] = v;
+            else out[seg_lane * Q + q] = v;
+        }
+        if (staged) {
+            __syncwarp(mask);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) out[q * SEG + seg_lane] = stage[q * SEG + seg_lane];
         }
     }
 }

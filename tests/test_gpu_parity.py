@@ -285,6 +285,24 @@ def test_streamed_wide_records(N, rows, cols, S, b, policy, every, tsize):
         assert_same(g.snapshot(), o.snapshot(), N)
 
 
+@pytest.mark.parametrize("N,rows,cols,every", [
+    (4, 5, 9, 1), (8, 5, 9, 1), (16, 3, 7, 1), (64, 3, 5, 1), (128, 3, 3, 1),  # staged stores
+    (8, 181, 182, 4), (16, 181, 182, 2), (64, 181, 182, 6),                     # direct: > 32,768 islands
+])
+def test_streamed_48_byte_stores(N, rows, cols, every):
+    """48-byte records leave through shared memory or directly by the generations to a launch and
+    the islands; missing last islands of a block on both."""
+    shape = RunShape(rows=rows, cols=cols, island_size=N, surface_sites=256, migrate_every=every,
+                     seed=77 + N, run_id=every, p_ben=0.05, p_del=0.05)
+    g, o = gpu_run(shape), oracle_for(shape)
+    g.resident_policy(1)  # GA_RESIDENT_OFF
+    for gens in (7, 6):
+        g.step(gens)
+        o.step(gens)
+    g.sync()
+    assert_same(g.snapshot(), o.snapshot(), N)
+
+
 @pytest.mark.parametrize("N,rows,cols,S,b,policy,every,tsize,model", [
     (128, 3, 7, 64, 1, "STEADY", 1, 5, 0), (128, 3, 3, 256, 1, "HYBRID", 4, 3, 0), (128, 1, 2, 128, 1, "STEADY", 16, 8, 0),
     (128, 2, 5, 32, 8, "TILTED", 0, 5, 0), (64, 5, 7, 64, 1, "STEADY", 4, 5, 0), (64, 3, 5, 8, 8, "TILTED", 16, 2, 0),
