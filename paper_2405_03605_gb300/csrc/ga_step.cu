@@ -6,8 +6,24 @@
 
 namespace ga {
 
-constexpr int kStepThreads = 256;
-constexpr int kStepWarps = kStepThreads / 32;
+constexpr int kUnitsThreads = 256;
+
+// Warps per block of the one-unit kernel.  Four: the warps of a block wait at its one barrier for
+// the warp that does the bookkeeping, and smaller blocks leave more of the others at work (4.2M
+// agents, a migration per generation, us a generation with 4 and 8 warps: 48-byte records,
+// islands of 8 69.6 and 74.5, of 32 63.9 and 67.4, of 128 66.7 and 71.5; 32-byte records, islands
+// of 32 46.6 and 49.3; 16-byte records, islands of 128 27.4 and 30.9).  Two is slower for most
+// (islands of 32, 4 generations to a launch: 26.6 against 23.7).  Eight for 16-byte records in
+// islands of 4 and 8, whose bookkeeping takes every lane of four warps or two (65,536 to 1M agents
+// 1 to 3% faster than with four).
+template <int N, int SW>
+constexpr int step_warps() { return N <= 8 && SW <= 2 ? 8 : 4; }
+
+// Blocks per SM asked of the compiler: 12 (40 registers) for 48-byte records with equal counters
+// in islands of 16 and 32, which take 44 to 46 unasked: 61.7 against 63.9 us a generation for 4.2M
+// agents in islands of 32, 15.5 against 15.9 for 1M.
+template <int N, int SW, int CF>
+constexpr int step_min_blocks() { return SW == 8 && CF == 0 && (N == 16 || N == 32) ? 12 : 1; }
 
 // Single run: per-run values and round keys are kernel parameters (constant bank).
 struct StepArgs {
@@ -16,10 +32,11 @@ struct StepArgs {
 };
 
 template <int N, int SW, int TS, int MODEL = 0, int CF = 1>
-__global__ void __launch_bounds__(kStepThreads) island_step_kernel(const StepArgs a)
+__global__ void __launch_bounds__((32 * step_warps<N, SW>()), (step_min_blocks<N, SW, CF>()))
+    island_step_kernel(const StepArgs a)
 {
     wait_previous_grid();
-    step_block<N, SW, TS, kStepWarps, MODEL, CF>(a.r, a.rk, blockIdx.x);
+    step_block<N, SW, TS, step_warps<N, SW>(), MODEL, CF>(a.r, a.rk, blockIdx.x);
 }
 
 // Multi-unit kernel (step_units in ga_island.cuh) for 16-byte records whose counters all
@@ -32,7 +49,7 @@ template <int N, int MODEL>
 constexpr int units_min_blocks() { return MODEL == 1 ? 4 : N >= 64 ? 6 : 8; }
 
 template <int N, int TS, int MODEL>
-__global__ void __launch_bounds__(kStepThreads, (units_min_blocks<N, MODEL>())) island_units_kernel(const StepArgs a)
+__global__ void __launch_bounds__(kUnitsThreads, (units_min_blocks<N, MODEL>())) island_units_kernel(const StepArgs a)
 {
     wait_previous_grid();
     step_units<N, TS, units_per_block<N>(), MODEL>(a.r, a.rk, blockIdx.x);
@@ -287,7 +304,7 @@ cudaError_t launch_island_step(ga_run *run, const void *src, void *dst, uint32_t
                                   static_cast<uint32_t>(run->cfg.seed >> 32)});
             const uint32_t blocks = (run->n_islands + islands_per_block - 1) / islands_per_block;
             run->launches += 1;
-            return launch_dependent(ku, blocks, kStepThreads, stream, a);
+            return launch_dependent(ku, blocks, kUnitsThreads, stream, a);
         }
     }
     StepKernel k =
@@ -302,10 +319,11 @@ cudaError_t launch_island_step(ga_run *run, const void *src, void *dst, uint32_t
     a.rk = round_keys(Key{static_cast<uint32_t>(run->cfg.seed),
                           static_cast<uint32_t>(run->cfg.seed >> 32)});
     const uint32_t N = run->cfg.island_size;
-    const uint32_t islands_per_block = kStepWarps * (N >= 32 ? 1u : 32u / N);
+    const uint32_t warps = N <= 8u && run->surface_words <= 2u ? step_warps<8, 2>() : step_warps<32, 2>();
+    const uint32_t islands_per_block = warps * (N >= 32 ? 1u : 32u / N);
     const uint32_t blocks = (run->n_islands + islands_per_block - 1) / islands_per_block;
     run->launches += 1;
-    return launch_dependent(k, blocks, kStepThreads, stream, a);
+    return launch_dependent(k, blocks, 32u * warps, stream, a);
 }
 
 cudaError_t launch_site_table(ga_run *run, uint32_t g0, uint32_t count, cudaStream_t stream)
