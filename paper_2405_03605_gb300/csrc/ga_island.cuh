@@ -572,7 +572,7 @@ __device__ __forceinline__ void step_block(const RunParams &p, const RoundKeys &
     // 48-byte records go out through shared memory (space whose contents have been read: the
     // island's part of the landing table, the warp's surfaces; else its own), 32 agents at a time
     // and each store a full run of 128-byte lines: a lane's own three stores leave every line to
-    // be filled by three instructions.  256 sites, a migration per generation, us a generation:
+    // be filled by three instructions.  256 sites, a migration per generation, us a generation (blocks of eight warps):
     // islands of 32: 2.78 against 3.16 for 65,536 agents, 16.7 against 18.6 for 1M, 66.1 against
     // 69.9 for 4.2M; of 64: 62.1 against 68.1; of 128: 70.3 against 76.4.  With several
     // generations to a launch the stores are few and the arithmetic bounds large runs, where the
