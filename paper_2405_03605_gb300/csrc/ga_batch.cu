@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(256, (N >= 64 ? 6 : 8)) batch_units_kernel(con
     // the unit loop unrolled for the compiled-in tournament size only: with the run's
     // parameters read from shared memory the unrolled run-time-size body spills (146.6 against
     // 152.2e9 agent-gens/s on the 256-run mix)
-    step_units<N, TS, units_per_block<N>(), 0, TS == 5>(s_r, a.rk, s_unit);
+    step_units<N, TS, units_per_block<N>(), 0, TS == 5, true>(s_r, a.rk, s_unit);
 }
 
 __global__ void batch_sites_kernel(const RunDesc *__restrict__ runs, uint32_t n_runs,

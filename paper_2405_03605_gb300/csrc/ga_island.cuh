@@ -572,14 +572,15 @@ __device__ __forceinline__ void step_block(const RunParams &p, const RoundKeys &
     // 48-byte records go out through shared memory (space whose contents have been read: the
     // island's part of the landing table, the warp's surfaces; else its own), 32 agents at a time
     // and each store a full run of 128-byte lines: a lane's own three stores leave every line to
-    // be filled by three instructions.  256 sites, a migration per generation, us a generation (blocks of eight warps):
-    // islands of 32: 2.78 against 3.16 for 65,536 agents, 16.7 against 18.6 for 1M, 66.1 against
-    // 69.9 for 4.2M; of 64: 62.1 against 68.1; of 128: 70.3 against 76.4.  With several
-    // generations to a launch the stores are few and the arithmetic bounds large runs, where the
-    // extra pass costs up to 4% (2 generations, islands of 32, 4.2M agents: 39.8 against 38.9;
-    // islands of 64: 37.3 against 39.4, even from 8 on); with at most 32,768 islands it still
-    // gains (262,144 agents, 4 generations: 2.15 against 2.26).  32-byte records, whose own stores
-    // fill whole sectors, are written directly: 53.6 us against 49.6 for 4.2M the other way.
+    // be filled by three instructions.  256 sites, a migration per generation, us a generation
+    // (blocks of eight warps): islands of 32: 2.78 against 3.16 for 65,536 agents, 16.7 against
+    // 18.6 for 1M, 66.1 against 69.9 for 4.2M; of 64: 62.1 against 68.1; of 128: 70.3 against
+    // 76.4.  With several generations to a launch the stores are few and the arithmetic bounds
+    // large runs, where the extra pass costs up to 4% (2 generations, islands of 32, 4.2M agents:
+    // 39.8 against 38.9; islands of 64: 37.3 against 39.4, even from 8 on); with at most 32,768
+    // islands it still gains (262,144 agents, 4 generations: 2.15 against 2.26).  32-byte records,
+    // whose own stores fill whole sectors, are written directly: 53.6 us against 49.6 for 4.2M the
+    // other way.
     constexpr bool kStaged = Q == 3, kOwn = kStaged && !kSlotTable && !kSurfaces;
     __shared__ uint4 s_out[kOwn ? WARPS : 1][kOwn ? SEG * Q : 1];
     uint4 *stage;
@@ -642,7 +643,10 @@ constexpr int units_per_block()
     return (256 / (4 * 8 * Shape<N>::P)) < 8 ? (256 / (4 * 8 * Shape<N>::P)) : 8;
 }
 
-template <int N, int TS, int U, int MODEL = 0, bool UNROLL = true>
+// ONE: every launch runs one generation (a batch's), so nothing of the later ones is compiled: with
+// the loop and its lookups there a batch of 10 runs, mostly islands of 64, took 3,650 us for 119
+// generations against 3,300 before the lookups.
+template <int N, int TS, int U, int MODEL = 0, bool UNROLL = true, bool ONE = false>
 __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &rk, uint32_t blk)
 {
     constexpr int SW = 2, LW = 4, WARPS = 8;
@@ -725,7 +729,7 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
     // traits through shared memory from a launch's second generation on (4.2M agents in islands of
     // 64, migration every 16 generations: 19.9 -> 17.6 us per generation; the first alone is 4%
     // slower with it)
-    constexpr bool kShared = N > 32;
+    constexpr bool kShared = N > 32 && !ONE;
     __shared__ int s_trait[kShared ? WARPS : 1][kShared ? 2 : 1][kShared ? N : 1];
     uint32_t turn = 0;
     auto lookup = [&]() {  // the next generation's set
@@ -888,7 +892,7 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
             rec[ag][3] = v.w;
         }
         reproduce<N, SW, TS, MODEL, 0, 1>(rec, w, p, rk, island, seg_lane, mask, p.g0, 0, dmask);
-        for (uint32_t it = 1; it < p.n_gens; ++it) {
+        for (uint32_t it = 1; !ONE && it < p.n_gens; ++it) {
             birth_draws<N>(w, p, rk, p.g0 + it, island, seg_lane);
             reproduce<N, SW, TS, MODEL, 0, 1>(rec, w, p, rk, island, seg_lane, mask, p.g0 + it, 0,
                                               gen_mask_at(p, it), nullptr, nullptr, lookup());
