@@ -96,7 +96,8 @@ __device__ __forceinline__ void stage_params(const BatchArgs &a, RunParams &s_r,
 }
 
 template <int N, int SW, int TS, int W, int CF = 1>
-__global__ void __launch_bounds__(W * 32) batch_step_kernel(const BatchArgs a)
+__global__ void __launch_bounds__((W * 32), (W == 4 && SW == 8 && CF == 0 && (N == 16 || N == 32) ? 12 : 1))
+    batch_step_kernel(const BatchArgs a)
 {
     __shared__ RunParams s_r;
     __shared__ uint32_t s_unit;
@@ -149,7 +150,10 @@ using BatchKernel = void (*)(BatchArgs);
 
 // Tournament size 5 (the paper's, Sec. 3) has its own instantiations; other sizes use the
 // kernels that read the size from the run.  CF = 0: classes whose members' counters all equal
-// their generations, compiled without the closed-form curation path (16-byte records only).
+// their generations, compiled without the closed-form curation path (wide records of islands of
+// 8 excepted).  24 runs of 256 sites, 256 generations, us a generation, with it and four warps
+// per block against the closed form and eight: islands of 16 25.4 against 25.9, of 32 47.8 against
+// 51.6, of 64 85.6 against 99.4; 128 sites, islands of 64 63.6 against 70.7.
 template <int N, int SW, int TS, int CF>
 BatchKernel pick_w(uint32_t warps)
 {
@@ -175,6 +179,10 @@ BatchKernel pick_sw(uint32_t sw, uint32_t ts, uint32_t warps, bool uniform)
             return ts == 5 ? batch_units_kernel<N, 5> : batch_units_kernel<N, 0>;
     }
     if (sw <= 2) return uniform ? pick_ts<N, 2, 0>(ts, warps) : pick_ts<N, 2, 1>(ts, warps);
+    if constexpr (N >= 16) {
+        if (uniform && sw <= 6) return pick_ts<N, 6, 0>(ts, warps);
+        if (uniform && sw <= 8) return pick_ts<N, 8, 0>(ts, warps);
+    }
     if (sw <= 6) return pick_ts<N, 6, 1>(ts, warps);
     if (sw <= 8) return pick_ts<N, 8, 1>(ts, warps);
     return nullptr;
@@ -198,7 +206,7 @@ struct Class {
     uint32_t island_size, sw_class, ts_class;
     uint64_t seed;
     bool uniform = false;  // every member's counters equal its generation (no closed form)
-    uint32_t warps = 8;
+    uint32_t warps = 8;  // before tuning; four for wide records, as the single-run kernel has it
     // islands one block covers: warps x islands per warp, or for the multi-unit kernel of
     // uniform 16-byte classes (8 warps, fixed) its units per block x islands per unit
     uint32_t per_block() const
@@ -363,7 +371,7 @@ int rebuild(ga_batch *b)
         const uint32_t swc = ga::sw_class(r->surface_words);
         const Key key = std::make_tuple(r->cfg.island_size, swc,
                                         ga::ts_class(r->cfg.tournament_size), r->cfg.seed,
-                                        swc == 2u && r->counters_uniform);
+                                        r->counters_uniform);
         auto it = index.find(key);
         if (it == index.end()) {
             ga::Class c;
@@ -372,6 +380,7 @@ int rebuild(ga_batch *b)
             c.ts_class = std::get<2>(key);
             c.seed = std::get<3>(key);
             c.uniform = std::get<4>(key);
+            c.warps = swc == 2u ? 8u : 4u;
             auto w = warps_of.find(key);
             if (w != warps_of.end()) c.warps = w->second;
             index[key] = b->classes.size();

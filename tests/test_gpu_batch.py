@@ -146,3 +146,34 @@ def test_large_member_steps_solo_bit_identical():
     o.step(13)
     assert_same(runs[1].snapshot(), o.snapshot(), 32)
     batch.close()
+
+
+@pytest.mark.parametrize("S,b,policy", [(256, 1, STEADY), (32, 8, TILTED), (128, 1, HYBRID)])
+def test_wide_classes_with_equal_and_mixed_counters(S, b, policy):
+    """32- and 48-byte members: classes of equal counters (no closed-form curation), beside members
+    loaded with different counters, each as when stepped alone, before and after tuning."""
+    from paper_2405_03605_gb300 import ga
+    shapes = [RunShape(rows=5, cols=7, island_size=N, tournament_size=ts, surface_sites=S,
+                       differentia_bits=b, curation=policy, migrate_every=k, p_ben=0.05, p_del=0.05,
+                       seed=4, run_id=i)
+              for i, (N, ts, k) in enumerate([(8, 5, 1), (16, 5, 1), (32, 5, 1), (64, 5, 4), (32, 3, 1), (64, 2, 1)])]
+    runs, alone = [gpu_run(s) for s in shapes], [gpu_run(s) for s in shapes]
+    batch = ga.Batch(runs)
+    batch.step(21)
+    batch.sync()
+    for r in alone:
+        r.step(21)
+    for r, a in list(zip(runs, alone))[2:4]:
+        rec = a.snapshot()
+        rec.view(np.uint32)[::3, 1] = 17
+        r.load(rec, 21)
+        a.load(rec, 21)
+    batch.step(18)
+    batch.autotune()
+    batch.step(9)
+    batch.sync()
+    for s, r, a in zip(shapes, runs, alone):
+        a.step(27)
+        a.sync()
+        assert np.array_equal(r.snapshot(), a.snapshot()), s
+    batch.close()
