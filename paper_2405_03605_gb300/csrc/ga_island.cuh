@@ -643,9 +643,12 @@ constexpr int units_per_block()
     return (256 / (4 * 8 * Shape<N>::P)) < 8 ? (256 / (4 * 8 * Shape<N>::P)) : 8;
 }
 
-// ONE: every launch runs one generation (a batch's), so nothing of the later ones is compiled: with
-// the loop and its lookups there a batch of 10 runs, mostly islands of 64, took 3,650 us for 119
-// generations against 3,300 before the lookups.
+// ONE: the launch runs one generation (a migration every generation, a batch), and nothing of the
+// later ones is compiled: fewer registers and no spills at the same blocks per SM, a shorter unrolled
+// loop, no lookups.  16.8M agents, us a generation: islands of 32 89.1 against 90.3, of 64 92.2
+// against 102.2, of 16 103.6 against 105.5, tournaments of three in islands of 32 86.8 against
+// 94.7, float model 136.1 against 146.6; a batch of 10 runs, mostly islands of 64, 3,121 against
+// 3,650 us for 119 generations.
 template <int N, int TS, int U, int MODEL = 0, bool UNROLL = true, bool ONE = false>
 __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &rk, uint32_t blk)
 {
@@ -840,7 +843,7 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
                     amount[ag] = (flags & kLowers) ? -drawn : drawn;
                 }
                 reproduce<N, SW, TS, 1, 0, 1, 1>(rec, w, p, rk, island, seg_lane, mask, p.g0, 0, dmask, amount, mutates);
-                for (uint32_t it = 1; it < p.n_gens; ++it) {
+                for (uint32_t it = 1; !ONE && it < p.n_gens; ++it) {
                     birth_draws<N>(w, p, rk, p.g0 + it, island, seg_lane);
                     reproduce<N, SW, TS, 1, 0, 1>(rec, w, p, rk, island, seg_lane, mask, p.g0 + it, 0,
                                                   gen_mask_at(p, it), nullptr, nullptr, lookup());

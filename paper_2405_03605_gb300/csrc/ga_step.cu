@@ -41,18 +41,18 @@ __global__ void __launch_bounds__((32 * step_warps<N, SW>()), (step_min_blocks<N
 
 // Multi-unit kernel (step_units in ga_island.cuh) for 16-byte records whose counters all
 // equal the generation, islands of 16, 32 or 64 agents, any tournament size, both genome
-// models; TS = 0 reads the tournament size from the run.
+// models; TS = 0 reads the tournament size from the run; ONE: launches of one generation.
 // Resident blocks per SM asked of the compiler: 8 (32 registers) below 64 agents; the two
 // agents per lane of 64-agent islands need 40 registers (6 blocks).  The float model, 4: its
 // deviates need 64 (50 generations of 16.8M agents: 7,433 us; 7,638 with 5 blocks, 7,865 with 3).
 template <int N, int MODEL>
 constexpr int units_min_blocks() { return MODEL == 1 ? 4 : N >= 64 ? 6 : 8; }
 
-template <int N, int TS, int MODEL>
+template <int N, int TS, int MODEL, bool ONE>
 __global__ void __launch_bounds__(kUnitsThreads, (units_min_blocks<N, MODEL>())) island_units_kernel(const StepArgs a)
 {
     wait_previous_grid();
-    step_units<N, TS, units_per_block<N>(), MODEL>(a.r, a.rk, blockIdx.x);
+    step_units<N, TS, units_per_block<N>(), MODEL, true, ONE>(a.r, a.rk, blockIdx.x);
 }
 
 // Every record becomes the founder: trait 0, counter 0, surface word w = word 0 of
@@ -129,6 +129,20 @@ StepKernel pick_fitness(uint32_t surface_words, uint32_t tsize)
 {
     if (surface_words > 2) return nullptr;
     return tsize == 5 ? island_step_kernel<N, 2, 5, 1> : island_step_kernel<N, 2, 0, 1>;
+}
+
+// Launches of one generation have a kernel of their own (see step_units).
+template <int N, int TS, int MODEL>
+StepKernel units_one(bool one)
+{
+    return one ? island_units_kernel<N, TS, MODEL, true> : island_units_kernel<N, TS, MODEL, false>;
+}
+
+template <int N>
+StepKernel pick_units(uint32_t tsize, bool fitness, bool one)
+{
+    if (fitness) return tsize == 5 ? units_one<N, 5, 1>(one) : units_one<N, 0, 1>(one);
+    return tsize == 5 ? units_one<N, 5, 0>(one) : units_one<N, 0, 0>(one);
 }
 
 // Kernels without the closed-form curation path, for launches whose counters all equal the
@@ -281,18 +295,15 @@ cudaError_t launch_island_step(ga_run *run, const void *src, void *dst, uint32_t
         uint32_t islands_per_block = 0;
         switch (N) {
         case 16:
-            ku = fit ? (ts == 5 ? island_units_kernel<16, 5, 1> : island_units_kernel<16, 0, 1>)
-                     : (ts == 5 ? island_units_kernel<16, 5, 0> : island_units_kernel<16, 0, 0>);
+            ku = pick_units<16>(ts, fit, n_gens == 1u);
             islands_per_block = units_per_block<16>() * 16;
             break;
         case 32:
-            ku = fit ? (ts == 5 ? island_units_kernel<32, 5, 1> : island_units_kernel<32, 0, 1>)
-                     : (ts == 5 ? island_units_kernel<32, 5, 0> : island_units_kernel<32, 0, 0>);
+            ku = pick_units<32>(ts, fit, n_gens == 1u);
             islands_per_block = units_per_block<32>() * 8;
             break;
         case 64:
-            ku = fit ? (ts == 5 ? island_units_kernel<64, 5, 1> : island_units_kernel<64, 0, 1>)
-                     : (ts == 5 ? island_units_kernel<64, 5, 0> : island_units_kernel<64, 0, 0>);
+            ku = pick_units<64>(ts, fit, n_gens == 1u);
             islands_per_block = units_per_block<64>() * 8;
             break;
         default: break;
