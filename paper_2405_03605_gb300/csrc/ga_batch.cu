@@ -114,9 +114,9 @@ __global__ void __launch_bounds__(256, (N >= 64 ? 6 : 8)) batch_units_kernel(con
     __shared__ RunParams s_r;
     __shared__ uint32_t s_unit;
     stage_params(a, s_r, s_unit);
-    // the unit loop unrolled for the compiled-in tournament size only: with the run's
-    // parameters read from shared memory the unrolled run-time-size body spills (146.6 against
-    // 152.2e9 agent-gens/s on the 256-run mix)
+    // the unit loop unrolled for the compiled-in tournament size only: the run-time-size classes run
+    // together and their unrolled bodies crowd the instruction cache (32-run mix, 256 generations:
+    // 15,960 against 14,080 us)
     step_units<N, TS, units_per_block<N>(), 0, TS == 5, true>(s_r, a.rk, s_unit);
 }
 

@@ -44,7 +44,8 @@ __global__ void __launch_bounds__((32 * step_warps<N, SW>()), (step_min_blocks<N
 // models; TS = 0 reads the tournament size from the run; ONE: launches of one generation.
 // Resident blocks per SM asked of the compiler: 8 (32 registers) below 64 agents; the two
 // agents per lane of 64-agent islands need 40 registers (6 blocks).  The float model, 4: its
-// deviates need 64 (50 generations of 16.8M agents: 7,433 us; 7,638 with 5 blocks, 7,865 with 3).
+// deviates need 64 (50 generations of 16.8M agents: 7,433 us; 7,638 with 5 blocks, 7,865 with 3; 6,900
+// since launches of one generation are compiled apart).
 template <int N, int MODEL>
 constexpr int units_min_blocks() { return MODEL == 1 ? 4 : N >= 64 ? 6 : 8; }
 
