@@ -22,9 +22,9 @@
 //   4. lands the arrivals in its islands' records (shared memory) and reproduces.
 //
 // Mailboxes: a 16-byte record is its own ready flag (its counter is g); wider records travel as
-// three 16-byte chunks of three words and the generation, their counter being g.  Each chunk is
-// one 128-bit relaxed store and load at GPU scope, so it is seen whole or not at all.  They are
-// double-buffered by migration parity: a sender can only overwrite a chunk after it has received
+// three 16-byte chunks of three words and the generation, their counter being g (32-byte records:
+// the third chunk one word and the generation three times).  Each chunk is one 128-bit relaxed
+// store and load at GPU scope, so it is seen whole or not at all.  They are double-buffered by migration parity: a sender can only overwrite a chunk after it has received
 // the receiver's next push, which the receiver makes after reading that chunk.  Every island
 // pushes before it polls and the cooperative launch keeps every warp resident, so each poll is
 // answered once the neighbour reaches the same generation.  Runs without mailboxes in their
@@ -80,7 +80,10 @@ __device__ __forceinline__ unsigned long long global_ns()
 }
 
 // 128-bit relaxed accesses at GPU scope, each one memory operation: the reader sees all of a
-// 16-byte chunk or none of it.
+// 16-byte chunk or none of it.  The reader has to use all four words: of a load with unused words
+// only the others are loaded, and no longer in one access (32-byte records whose third chunk
+// carried two unused words arrived with that chunk's new generation and its old first word some
+// three times in 100,000 migrants).
 __device__ __forceinline__ uint4 load128(const uint4 *p)
 {
     unsigned long long lo, hi;
@@ -240,7 +243,7 @@ __global__ void __launch_bounds__(32, 20) resident_kernel(const ResidentArgs a)
                         if constexpr (Q == 3) r2 = r[2];
                         store128(box, make_uint4(r0.x, r0.z, r0.w, g));
                         store128(box + 1, make_uint4(r1.x, r1.y, r1.z, g));
-                        store128(box + 2, make_uint4(r1.w, r2.x, r2.y, g));
+                        store128(box + 2, Q == 3 ? make_uint4(r1.w, r2.x, r2.y, g) : make_uint4(r1.w, g, g, g));
                     }
                 }
             }
@@ -259,7 +262,7 @@ __global__ void __launch_bounds__(32, 20) resident_kernel(const ResidentArgs a)
                 };
                 auto arrived = [&]() {
                     if constexpr (C == 1) return in[0].y == g;
-                    else return in[0].w == g && in[1].w == g && in[2].w == g;
+                    else return in[0].w == g && in[1].w == g && in[2].w == g && (Q == 3 || (in[2].y == g && in[2].z == g));
                 };
                 // while the pushes and the first reads travel: the next migration's draws and the
                 // first islands' birth draws.  An arrival is read right after the pushes, and a
