@@ -131,7 +131,7 @@ constexpr uint32_t kResidentMaxIslands = 8192;
 constexpr uint32_t kResidentAutoGens = 4;
 size_t resident_state_bytes(uint32_t n_islands, uint32_t record_bytes);
 struct ResidentPlan {
-    uint32_t units, blocks;
+    uint32_t units, blocks, sms;
     size_t shared_bytes;
 };
 // What GA_RESIDENT_ON accepts and GA_RESIDENT_AUTO steps resident at any length: a synchronous run

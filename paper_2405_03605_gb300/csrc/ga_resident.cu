@@ -41,8 +41,8 @@
 // 1.15 us per generation), larger ones issue (9,991 islands of 32: 2.65 us per generation; 7.2 us
 // with one ordinary launch each, 4 with dependent ones).  Shapes, us for 250 generations of 9,991
 // islands of 16-byte and 5,893 of 48-byte records: one warp per block 665 and 562, four 707 and
-// 612 (what depends on the block alone stays in uniform registers); about 18 warps on an SM at
-// up to 96 registers against as many as 64 registers allow: 131,000 agents 1.7 and 2.3 us per
+// 612 (what depends on the block alone stays in uniform registers); 18 to 20 warps on an SM at up
+// to 96 registers against as many as 64 registers allow: 131,000 agents 1.7 and 2.3 us per
 // generation (the bookkeeping of one island takes a quarter of a warp's lanes), 262,000 2.4 and
 // 2.9.
 #include "ga_device.cuh"
@@ -56,9 +56,30 @@ RunParams run_params(const ga_run *run, const void *src, void *dst, uint32_t g0,
 
 namespace {
 
-
-// Warps per SM that a run is spread over, while its islands per warp allow it.
-constexpr uint32_t kWarpsPerSm = 18;
+// Units per warp: as few as keep an SM's warps to a limit, more where they don't fit at once.  An SM
+// has four schedulers, so a generation lengthens where a sixth warp falls to one of them: the limit
+// is 20.  Us per generation with one unit to a warp and with two, on either side of it (2,916 and
+// 3,080 islands of 32): float model 2.23 / 2.26 and 2.57 / 2.28, every 4 generations 1.31 / 1.56 and
+// 1.59 / 1.56; trait model every 4 0.76 / 0.77 and 0.90 / 0.77.  (A limit of 18 takes two from 2,737
+// on: 1.55 for the float model every 4, which took 1.41 with a warp to every island.)  But
+//   - float model, and islands of 16, with tournaments of run-time size and several generations to
+//     a migration: a unit's work is long, so one to a warp whatever the registers allow (25 to 28
+//     warps): 3,403 units 1.71 / 1.82 every 4, 1.54 / 1.59 every 16;
+//   - 16-byte trait records in islands of 32 or 64, tournaments of 5, a migration in one or two
+//     generations: so short that from 16 warps on two to a warp are faster, as the bookkeeping of
+//     one fills few of a warp's lanes: 2,500 and 2,704 islands of 32 1.62 / 1.55 and 1.67 / 1.57, of 64
+//     2.23 / 2.04, every 2 1.06 / 1.03.
+uint32_t units_per_warp(const ga_run *run, uint32_t n_units, uint32_t sms)
+{
+    const bool five = run->cfg.tournament_size == 5u, fit = run->cfg.model == GA_MODEL_FITNESS;
+    const uint32_t N = run->cfg.island_size, k = run->per_neighbor ? run->every_k : 0xFFFFFFFFu;
+    uint32_t single = 20u;
+    if (!five && k > 1u && (fit || N == 16u)) single = 28u;
+    else if (five && k <= 2u && !fit && N >= 32u && run->record_bytes == 16u) single = 16u;
+    if (n_units <= single * sms) return 1u;
+    const uint32_t units = (n_units + 20u * sms - 1u) / (20u * sms);
+    return units < 2u ? 2u : units;
+}
 
 struct ResidentArgs {
     RunParams r;
@@ -137,9 +158,11 @@ __host__ __device__ constexpr uint32_t warp_bytes(uint32_t islands)
 }
 
 // N, SW, TS, MODEL: island size, surface words, tournament size (0: read from the run) and genome
-// model, as in step_block; IV: migrations more than a generation apart.
-template <int N, int SW, int TS, int MODEL, bool IV>
-__global__ void __launch_bounds__(32, 20) resident_kernel(const ResidentArgs a)
+// model, as in step_block; IV: migrations more than a generation apart.  WARPS: resident warps per SM
+// asked of the compiler: 20 (96 registers), or 28 (72, a few spilled) for float runs in islands of 16
+// that need them (see pick_ts; 40,000 agents do not: 1.09 against 1.05 us every 4 generations).
+template <int N, int SW, int TS, int MODEL, bool IV, int WARPS = 20>
+__global__ void __launch_bounds__(32, WARPS) resident_kernel(const ResidentArgs a)
 {
     constexpr int A = Shape<N>::A, P = Shape<N>::P, SEG = Shape<N>::SEG;
     constexpr int LW = Record<SW>::LW, Q = Record<SW>::Q, C = Record<SW>::C;
@@ -409,11 +432,16 @@ ResidentPick picked(ResidentKernel k)
     return m;
 }
 
-// Tournament size 5 (the paper's) is compiled in; other sizes are read from the run.
+// Tournament size 5 (the paper's) is compiled in; other sizes are read from the run.  dense: 21 to 28
+// warps per SM with one unit each (float model, islands of 16, every 4 generations: 110,000 agents
+// 1.67 against 1.72 us per generation with the 96-register kernel, 131,072, where that one takes two
+// units to a warp, 1.96 against 2.12; every 16 1.84 against 1.90).
 template <int N, int SW, int MODEL = 0>
-ResidentPick pick_ts(uint32_t tsize, bool intervals)
+ResidentPick pick_ts(uint32_t tsize, bool intervals, bool dense = false)
 {
     if constexpr (SW == 2) {
+        if constexpr (N == 16 && MODEL == 1)
+            if (intervals && dense && tsize != 5u) return picked<N, SW>(resident_kernel<N, SW, 0, MODEL, true, 28>);
         if (intervals)
             return picked<N, SW>(tsize == 5u ? resident_kernel<N, SW, 5, MODEL, true>
                                              : resident_kernel<N, SW, 0, MODEL, true>);
@@ -425,11 +453,11 @@ ResidentPick pick_ts(uint32_t tsize, bool intervals)
 // The float-fitness model: 16-byte records, islands of 16 to 64 agents.  32-byte records: not
 // for islands of 8, whose mailboxes would not fit in the place of their records.
 template <int N>
-ResidentPick pick_n(uint32_t surface_words, uint32_t model, uint32_t tsize, bool intervals)
+ResidentPick pick_n(uint32_t surface_words, uint32_t model, uint32_t tsize, bool intervals, bool dense = false)
 {
     if (model == GA_MODEL_FITNESS) {
         if constexpr (N >= 16)
-            if (surface_words <= 2u) return pick_ts<N, 2, 1>(tsize, intervals);
+            if (surface_words <= 2u) return pick_ts<N, 2, 1>(tsize, intervals, dense);
         return ResidentPick();
     }
     if (surface_words <= 2u) return pick_ts<N, 2>(tsize, intervals);
@@ -440,13 +468,13 @@ ResidentPick pick_n(uint32_t surface_words, uint32_t model, uint32_t tsize, bool
     return pick_ts<N, 8>(tsize, intervals);
 }
 
-ResidentPick pick(const ga_run *run)
+ResidentPick pick(const ga_run *run, uint32_t sms)
 {
     const uint32_t sw = run->surface_words, model = run->cfg.model, ts = run->cfg.tournament_size;
     const bool iv = run->per_neighbor == 0u || run->every_k > 1u;
     switch (run->cfg.island_size) {
     case 8: return pick_n<8>(sw, model, ts, iv);
-    case 16: return pick_n<16>(sw, model, ts, iv);
+    case 16: return pick_n<16>(sw, model, ts, iv, run->n_islands > 40u * sms && run->n_islands <= 56u * sms);
     case 32: return pick_n<32>(sw, model, ts, iv);
     case 64: return pick_n<64>(sw, model, ts, iv);
     default: return ResidentPick();
@@ -525,22 +553,24 @@ bool resident_pays(const ga_run *run)
 bool resident_plan(const ga_run *run, ResidentPlan &plan)
 {
     if (run->cfg.mode != GA_SYNC || !run->counters_uniform) return false;
-    const ResidentPick m = pick(run);
-    if (!m.k) return false;
     int dev = 0, sms = 0, smem = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-        cudaFuncSetAttribute(reinterpret_cast<const void *>(m.k),
+        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    plan.sms = static_cast<uint32_t>(sms);
+    const ResidentPick m = pick(run, plan.sms);
+    if (!m.k) return false;
+    if (cudaFuncSetAttribute(reinterpret_cast<const void *>(m.k),
                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     if (static_cast<uint64_t>(run->n_islands) * m.bytes_per_island > static_cast<uint64_t>(sms) * smem) return false;
-    // islands per warp for about kWarpsPerSm warps on an SM, more where they don't fit at once
     const uint32_t n_units = (run->n_islands + m.islands_per_unit - 1u) / m.islands_per_unit;
-    const uint32_t want = static_cast<uint32_t>(sms) * kWarpsPerSm;
-    for (uint32_t units = (n_units + want - 1u) / want;; ++units) {
+    for (uint32_t units = units_per_warp(run, n_units, plan.sms);; ++units) {
         const size_t bytes = static_cast<size_t>(units) * m.islands_per_unit * m.bytes_per_island;
         if (bytes > static_cast<size_t>(smem)) return false;
         int per_sm = 0;
@@ -549,7 +579,7 @@ bool resident_plan(const ga_run *run, ResidentPlan &plan)
             return false;
         }
         const uint32_t blocks = (n_units + units - 1u) / units;
-        if (blocks <= static_cast<uint32_t>(sms) * static_cast<uint32_t>(per_sm)) {
+        if (blocks <= plan.sms * static_cast<uint32_t>(per_sm)) {
             plan.units = units;
             plan.blocks = blocks;
             plan.shared_bytes = bytes;
@@ -561,7 +591,7 @@ bool resident_plan(const ga_run *run, ResidentPlan &plan)
 cudaError_t launch_resident(ga_run *run, const ResidentPlan &plan, const void *src, void *dst, uint32_t g0,
                             uint32_t n_gens, cudaStream_t stream)
 {
-    const ResidentPick m = pick(run);
+    const ResidentPick m = pick(run, plan.sms);
     if (!m.k) return cudaErrorInvalidValue;
     ResidentArgs a;
     a.r = run_params(run, src, dst, g0, n_gens, false);
