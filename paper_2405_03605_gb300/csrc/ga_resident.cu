@@ -57,11 +57,12 @@ RunParams run_params(const ga_run *run, const void *src, void *dst, uint32_t g0,
 namespace {
 
 // Units per warp: as few as keep an SM's warps to a limit, more where they don't fit at once.  An SM
-// has four schedulers, so a generation lengthens where a sixth warp falls to one of them: the limit
-// is 20.  Us per generation with one unit to a warp and with two, on either side of it (2,916 and
-// 3,080 islands of 32): float model 2.23 / 2.26 and 2.57 / 2.28, every 4 generations 1.31 / 1.56 and
-// 1.59 / 1.56; trait model every 4 0.76 / 0.77 and 0.90 / 0.77.  (A limit of 18 takes two from 2,737
-// on: 1.55 for the float model every 4, which took 1.41 with a warp to every island.)  But
+// has four schedulers, so a generation lengthens where a sixth warp falls to one of them: with one
+// unit to a warp the limit is 20.  Us per generation with one unit to a warp and with two, on
+// either side of it (2,916 and 3,080 islands of 32): float model 2.23 / 2.26 and 2.57 / 2.28, every 4
+// generations 1.31 / 1.56 and 1.59 / 1.56; trait model every 4 0.76 / 0.77 and 0.90 / 0.77.  (A limit of
+// 18 takes two from 2,737 on: 1.55 for the float model every 4, which took 1.41 with a warp to
+// every island.)  But
 //   - float model, and islands of 16, with tournaments of run-time size and several generations to
 //     a migration: a unit's work is long, so one to a warp whatever the registers allow (25 to 28
 //     warps): 3,403 units 1.71 / 1.82 every 4, 1.54 / 1.59 every 16;
@@ -69,6 +70,8 @@ namespace {
 //     generations: so short that from 16 warps on two to a warp are faster, as the bookkeeping of
 //     one fills few of a warp's lanes: 2,500 and 2,704 islands of 32 1.62 / 1.55 and 1.67 / 1.57, of 64
 //     2.23 / 2.04, every 2 1.06 / 1.03.
+// With more units to a warp, 18: 14,062 islands of 32 5 or 6 to a warp (18.5 and 15.4 warps) 3.42 and
+// 3.12, float model 6.14 and 5.75; 48-byte records in islands of 16 6.3 and 5.7.
 uint32_t units_per_warp(const ga_run *run, uint32_t n_units, uint32_t sms)
 {
     const bool five = run->cfg.tournament_size == 5u, fit = run->cfg.model == GA_MODEL_FITNESS;
@@ -77,7 +80,7 @@ uint32_t units_per_warp(const ga_run *run, uint32_t n_units, uint32_t sms)
     if (!five && k > 1u && (fit || N == 16u)) single = 28u;
     else if (five && k <= 2u && !fit && N >= 32u && run->record_bytes == 16u) single = 16u;
     if (n_units <= single * sms) return 1u;
-    const uint32_t units = (n_units + 20u * sms - 1u) / (20u * sms);
+    const uint32_t units = (n_units + 18u * sms - 1u) / (18u * sms);
     return units < 2u ? 2u : units;
 }
 
