@@ -527,30 +527,38 @@ bool resident_eligible(const ga_run *run)
 }
 
 // A streamed launch covers a migration interval of k generations, so resident launches save
-// fewer launches as k grows, while the streamed kernels keep three times the warps on an SM.  Us
-// per generation, streamed / resident, on either side of each line (16-byte records but for W,
-// 48-byte ones, and X, 32-byte ones; thousands of agents):
-//   k = 1   N = 8: 131 2.40 / 2.21, 196 3.25 / 3.33;  16: 320 4.3 / 3.4, 400 4.4 / 4.7;
-//           32: 1,300 8.9 / 8.5, 1,600 10.3 / 10.9;  64: 1,300 12.2 / 9.9, 1,600 12.2 / 12.7
-//   k = 2   8: 98 1.37 / 1.35, 131 1.53 / 1.56;  16: 262 2.5 / 2.4, 400 3.2 / 3.9;
-//           32: 500 3.9 / 3.6, 600 3.9 / 4.1;  64: 1,300 10.7 / 10.0, 1,600 10.8 / 12.5;
-//           X: 600 4.4 / 4.3, 800 5.6 / 6.0
-//   k = 4   8: 65 0.78 / 0.72, 98 0.92 / 0.94;  16: 196 1.86 / 1.55, 262 1.88 / 1.99;
-//           32: 400 3.2 / 2.7, 500 3.2 / 3.2;  64: 600 4.3 / 3.9, 1,000 6.7 / 7.8;
-//           W: 196 1.59 / 1.49, 400 2.7 / 2.8;  X: 131 1.14 / 1.15
-//   k = 16  8: 16 0.34 / 0.32, 65 0.44 / 0.51;  16: 196 1.4 / 1.3, 262 1.4 / 1.7;
-//           32: 400 2.7 / 2.4, 500 2.7 / 2.9;  64: 400 3.7 / 3.3, 500 3.7 / 3.8;
-//           W: 16 0.38 / 0.41
+// fewer launches as k grows, while the streamed kernels keep three times the warps on an SM.  The
+// most agents, in thousands, up to which they are faster; rows: islands of 8, 16, 32, 64; columns:
+// 16-byte trait records, the float model, 32-byte, 48-byte records.  Streamed / resident, us per
+// generation (the slower of tournaments of 5 and 3) on either side of some lines:
+//   k = 1   16-byte: 16: 350 4.3 / 3.6, 400 4.1 / 4.7; 32: 1,000 7.1 / 6.9, 1,100 7.1 / 7.7; 64: 1,100 8.5 / 8.5
+//           float: 32: 750 9.0 / 8.8, 800 9.1 / 10.6;  32-byte: 16: 700 8.94 / 8.93, 1,000 12.0 / 31
+//           48-byte: 16: 650 10.2 / 8.8, 700 10.7 / 28 (too few warps fit); 64: 700 10.4 / 7.5
+//   k = 2   48-byte: 16: 600 5.85 / 5.77, 700 6.5 / 22; 32: 600 5.45 / 4.37;  32-byte: 64: 450 3.9 / 3.9
+//   k = 4   32-byte: 16: 65 1.00, 98 0.91 of the streamed rate; 32: 98 1.02, 131 0.92; 64: 114 1.05, 131 0.95
+//   k = 6   48-byte: 32: 150 1.02, 175 0.93; 64: 114 0.97 to 1.06, 131 0.89 to 0.98;  k = 8: 32: 65 0.99, 81 0.96
+struct ResidentLines {
+    uint32_t every;  // up to this migration interval
+    uint16_t most[4][4];
+};
+constexpr ResidentLines kResidentLines[] = {
+    {1u, {{150, 0, 0, 150}, {380, 375, 700, 650}, {1000, 750, 1100, 700}, {1400, 1400, 1000, 700}}},
+    {2u, {{99, 0, 0, 99}, {300, 275, 300, 600}, {500, 500, 550, 600}, {1400, 1400, 450, 600}}},
+    {4u, {{66, 0, 0, 66}, {200, 200, 66, 150}, {400, 400, 99, 200}, {600, 600, 115, 150}}},
+    {6u, {{66, 0, 0, 66}, {200, 200, 0, 50}, {400, 400, 50, 150}, {600, 600, 66, 115}}},
+    {8u, {{66, 0, 0, 0}, {200, 200, 0, 0}, {400, 400, 0, 66}, {600, 600, 0, 33}}},
+    {~0u, {{0, 0, 0, 0}, {200, 200, 0, 0}, {400, 400, 0, 0}, {400, 400, 0, 0}}},
+};
+
 bool resident_pays(const ga_run *run)
 {
-    const uint32_t k = run->per_neighbor ? run->every_k : 0xFFFFFFFFu;
-    const uint32_t N = run->cfg.island_size, bytes = run->record_bytes;
-    uint32_t most = 0;  // agents
-    if (k == 1u) most = N == 8u ? 150000u : N == 16u && bytes == 16u ? 380000u : 1400000u;
-    else if (k == 2u) most = N == 8u ? 98304u : bytes != 16u ? 600000u : N == 16u ? 300000u : N == 32u ? 500000u : 1400000u;
-    else if (k <= 8u) most = N == 8u ? 65536u : bytes == 32u ? 131072u : bytes == 48u || N == 16u ? 200000u : N == 32u ? 400000u : 600000u;
-    else if (N >= 16u && bytes == 16u) most = N == 16u ? 200000u : 400000u;
-    return run->n_agents <= most;
+    const uint32_t N = run->cfg.island_size, k = run->per_neighbor ? run->every_k : ~0u;
+    if (N < 8u || N > 64u) return false;
+    const ResidentLines *row = kResidentLines;
+    while (k > row->every) ++row;
+    const uint32_t kind = run->cfg.model == GA_MODEL_FITNESS ? 1u : run->record_bytes == 16u ? 0u : run->record_bytes / 16u;
+    const uint32_t size = N == 8u ? 0u : N == 16u ? 1u : N == 32u ? 2u : 3u;
+    return run->n_agents <= row->most[size][kind] * 1000u;
 }
 
 bool resident_plan(const ga_run *run, ResidentPlan &plan)
