@@ -649,7 +649,9 @@ constexpr int units_per_block()
 // against 102.2, of 16 103.6 against 105.5, tournaments of three in islands of 32 86.8 against
 // 94.7, float model 136.1 against 146.6; a batch of 10 runs, mostly islands of 64, 3,121 against
 // 3,650 us for 119 generations.
-template <int N, int TS, int U, int MODEL = 0, bool UNROLL = true, bool ONE = false>
+// QUEUE: the first generation's mutating births of the float model go through a queue (below); without
+// it every generation draws them in place.
+template <int N, int TS, int U, int MODEL = 0, bool UNROLL = true, bool ONE = false, bool QUEUE = MODEL == 1>
 __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &rk, uint32_t blk)
 {
     constexpr int SW = 2, LW = 4, WARPS = 8;
@@ -732,7 +734,9 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
     // traits through shared memory from a launch's second generation on (4.2M agents in islands of
     // 64, migration every 16 generations: 19.9 -> 17.6 us per generation; the first alone is 4%
     // slower with it)
-    constexpr bool kShared = N > 32 && !ONE;
+    // (slower for the float model's plain kernel with tournaments of run-time size: 131,072 to 500,000
+    // agents without migration 10.1 against 9.9 us)
+    constexpr bool kShared = N > 32 && !ONE && (MODEL == 0 || QUEUE || TS == 5);
     __shared__ int s_trait[kShared ? WARPS : 1][kShared ? 2 : 1][kShared ? N : 1];
     uint32_t turn = 0;
     auto lookup = [&]() {  // the next generation's set
@@ -747,7 +751,7 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
     // shared-memory offsets of each unit and the loop control become constants (94.2 against
     // 101.7 us per generation of 16.8M agents with the loop kept rolled; 3-10% on the other
     // island and tournament sizes, results identical)
-    if constexpr (MODEL == 1) {
+    if constexpr (QUEUE) {
         // Float model.  About a third of the births mutate, and a warp in which any lane does would
         // run the second Philox call and the normal deviate (230 instructions) for all 32.  So a
         // warp draws eight births per lane at a time (four where the shared memory or the block's

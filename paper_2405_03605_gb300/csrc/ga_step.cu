@@ -43,17 +43,17 @@ __global__ void __launch_bounds__((32 * step_warps<N, SW>()), (step_min_blocks<N
 // equal the generation, islands of 16, 32 or 64 agents, any tournament size, both genome
 // models; TS = 0 reads the tournament size from the run; ONE: launches of one generation.
 // Resident blocks per SM asked of the compiler: 8 (32 registers) below 64 agents; the two
-// agents per lane of 64-agent islands need 40 registers (6 blocks).  The float model, 4: its
-// deviates need 64 (50 generations of 16.8M agents: 7,433 us; 7,638 with 5 blocks, 7,865 with 3; 6,900
-// since launches of one generation are compiled apart).
-template <int N, int MODEL>
-constexpr int units_min_blocks() { return MODEL == 1 ? 4 : N >= 64 ? 6 : 8; }
+// agents per lane of 64-agent islands need 40 registers (6 blocks).  The float model's queue needs
+// 64: 4 (50 generations of 16.8M agents: 7,433 us; 7,638 with 5 blocks, 7,865 with 3; 6,900 since
+// launches of one generation are compiled apart).
+template <int N, bool QUEUE>
+constexpr int units_min_blocks() { return QUEUE ? 4 : N >= 64 ? 6 : 8; }
 
-template <int N, int TS, int MODEL, bool ONE>
-__global__ void __launch_bounds__(kUnitsThreads, (units_min_blocks<N, MODEL>())) island_units_kernel(const StepArgs a)
+template <int N, int TS, int MODEL, bool ONE, bool QUEUE = MODEL == 1>
+__global__ void __launch_bounds__(kUnitsThreads, (units_min_blocks<N, QUEUE>())) island_units_kernel(const StepArgs a)
 {
     wait_previous_grid();
-    step_units<N, TS, units_per_block<N>(), MODEL, true, ONE>(a.r, a.rk, blockIdx.x);
+    step_units<N, TS, units_per_block<N>(), MODEL, true, ONE, QUEUE>(a.r, a.rk, blockIdx.x);
 }
 
 // Every record becomes the founder: trait 0, counter 0, surface word w = word 0 of
@@ -132,18 +132,36 @@ StepKernel pick_fitness(uint32_t surface_words, uint32_t tsize)
     return tsize == 5 ? island_step_kernel<N, 2, 5, 1> : island_step_kernel<N, 2, 0, 1>;
 }
 
+// Generations to a launch from which on the float model's kernel without the queue is faster: the queue
+// shortens the first generation alone, and the registers it takes halve the warps on an SM in the
+// later ones.  With the queue and without, 2.5M agents, us per generation:
+//   tournaments of 5   16 agents: 6 23.07 / 23.14, 8 22.75 / 22.42, none 22.02 / 20.74;  32: 8 24.62 / 24.78,
+//                      16 24.57 / 24.09, none 24.47 / 23.43;  64: 16 30.36 / 30.65, none 30.22 / 30.21
+//   of 3               16: 4 24.29 / 24.67, 6 23.83 / 23.68, none 22.74 / 21.44;  32: 2 27.69 / 28.45,
+//                      4 26.58 / 25.88, none 25.46 / 23.43;  64: 16 31.88 / 31.24 (5M agents 54.8 / 57.5), none
+//                      31.78 / 30.72 (54.5 / 55.4; 500,000 10.6 / 10.1)
+template <int N, int TS>
+constexpr uint32_t plain_from()
+{
+    if (TS == 5) return N == 16 ? 8u : N == 32 ? 16u : kMaxGensPerLaunch + 1u;
+    return N == 16 ? 6u : N == 32 ? 4u : 32u;
+}
+
 // Launches of one generation have a kernel of their own (see step_units).
 template <int N, int TS, int MODEL>
-StepKernel units_one(bool one)
+StepKernel units_of(uint32_t n_gens)
 {
-    return one ? island_units_kernel<N, TS, MODEL, true> : island_units_kernel<N, TS, MODEL, false>;
+    if (n_gens == 1u) return island_units_kernel<N, TS, MODEL, true>;
+    if constexpr (MODEL == 1 && plain_from<N, TS>() <= kMaxGensPerLaunch)
+        if (n_gens >= plain_from<N, TS>()) return island_units_kernel<N, TS, MODEL, false, false>;
+    return island_units_kernel<N, TS, MODEL, false>;
 }
 
 template <int N>
-StepKernel pick_units(uint32_t tsize, bool fitness, bool one)
+StepKernel pick_units(uint32_t tsize, bool fitness, uint32_t n_gens)
 {
-    if (fitness) return tsize == 5 ? units_one<N, 5, 1>(one) : units_one<N, 0, 1>(one);
-    return tsize == 5 ? units_one<N, 5, 0>(one) : units_one<N, 0, 0>(one);
+    if (fitness) return tsize == 5 ? units_of<N, 5, 1>(n_gens) : units_of<N, 0, 1>(n_gens);
+    return tsize == 5 ? units_of<N, 5, 0>(n_gens) : units_of<N, 0, 0>(n_gens);
 }
 
 // Kernels without the closed-form curation path, for launches whose counters all equal the
@@ -296,15 +314,15 @@ cudaError_t launch_island_step(ga_run *run, const void *src, void *dst, uint32_t
         uint32_t islands_per_block = 0;
         switch (N) {
         case 16:
-            ku = pick_units<16>(ts, fit, n_gens == 1u);
+            ku = pick_units<16>(ts, fit, n_gens);
             islands_per_block = units_per_block<16>() * 16;
             break;
         case 32:
-            ku = pick_units<32>(ts, fit, n_gens == 1u);
+            ku = pick_units<32>(ts, fit, n_gens);
             islands_per_block = units_per_block<32>() * 8;
             break;
         case 64:
-            ku = pick_units<64>(ts, fit, n_gens == 1u);
+            ku = pick_units<64>(ts, fit, n_gens);
             islands_per_block = units_per_block<64>() * 8;
             break;
         default: break;
