@@ -737,11 +737,12 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
     // (slower for the float model's plain kernel with tournaments of run-time size: 131,072 to 500,000
     // agents without migration 10.1 against 9.9 us)
     constexpr bool kShared = N > 32 && !ONE && (MODEL == 0 || QUEUE || TS == 5);
-    __shared__ int s_trait[kShared ? WARPS : 1][kShared ? 2 : 1][kShared ? N : 1];
+    constexpr bool kOwnTraits = kShared && !QUEUE;
+    __shared__ int s_trait[kOwnTraits ? WARPS : 1][kOwnTraits ? 2 : 1][kOwnTraits ? N : 1];
     uint32_t turn = 0;
     auto lookup = [&]() {  // the next generation's set
         Lookup l;
-        if constexpr (kShared) l.traits = s_trait[warp][turn++ & 1u];
+        if constexpr (kOwnTraits) l.traits = s_trait[warp][turn++ & 1u];
         return l;
     };
 
@@ -766,6 +767,9 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
         __shared__ Kept s_kept[WARPS][NB][32];       // tournament words, differentia, flags
         __shared__ float s_amount[WARPS][NB * 32];   // of mutating births
         __shared__ uint8_t s_queue[WARPS][NB * 32];  // mutating births: 32 b + lane
+        static_assert(sizeof(s_rec) + sizeof(s_imm) + sizeof(s_dir) + sizeof(s_trait) + sizeof(s_kept) + sizeof(s_amount) +
+                              sizeof(s_queue) <= 48u * 1024u,
+                      "static shared memory of a block");
         constexpr uint32_t kMutates = 1u << 16, kLowers = 1u << 17;
 #pragma unroll 1
         for (uint32_t gu = 0; gu < static_cast<uint32_t>(U); gu += GU) {
@@ -847,10 +851,15 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
                     amount[ag] = (flags & kLowers) ? -drawn : drawn;
                 }
                 reproduce<N, SW, TS, 1, 0, 1, 1>(rec, w, p, rk, island, seg_lane, mask, p.g0, 0, dmask, amount, mutates);
+                // the later generations' traits take the place of the unit's kept draws
+                static_assert(!kShared || sizeof(s_kept[0][0]) * A >= 2u * N * sizeof(int), "two sets of traits");
+                if constexpr (kShared) __syncwarp(mask);  // every lane has read its draws
                 for (uint32_t it = 1; !ONE && it < p.n_gens; ++it) {
+                    Lookup traits;
+                    if constexpr (kShared) traits.traits = reinterpret_cast<int *>(&s_kept[warp][h * A][0]) + (it & 1u) * N;
                     birth_draws<N>(w, p, rk, p.g0 + it, island, seg_lane);
                     reproduce<N, SW, TS, 1, 0, 1>(rec, w, p, rk, island, seg_lane, mask, p.g0 + it, 0,
-                                                  gen_mask_at(p, it), nullptr, nullptr, lookup());
+                                                  gen_mask_at(p, it), nullptr, nullptr, traits);
                 }
                 uint4 *dst = p.dst + static_cast<size_t>(first) * N + lane;
 #pragma unroll
