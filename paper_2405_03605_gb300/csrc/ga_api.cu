@@ -163,7 +163,13 @@ int step_run(ga_run *run, uint32_t n_gens, cudaStream_t stream, bool shared)
             run->sites_base = run->generation;
             const int rc = cuda_rc(launch_resident(run, plan, run->pop[run->cur], run->pop[run->cur ^ 1],
                                                    static_cast<uint32_t>(run->generation), chunk, stream));
-            if (rc != GA_OK) return rc;
+            if (rc != GA_OK) {
+                // a cooperative launch can be refused where the process may use fewer SMs than the
+                // device reports: nothing but the other buffer has been written, so AUTO streams
+                if (run->resident_mode == GA_RESIDENT_ON) return rc;
+                resident = false;
+                continue;
+            }
             run->cur ^= 1;
             run->generation += chunk;
             n_gens -= chunk;

@@ -631,7 +631,8 @@ cudaError_t launch_resident(ga_run *run, const ResidentPlan &plan, const void *s
     void *args[] = {&a};
     e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(m.k), dim3(plan.blocks), dim3(32),
                                     args, plan.shared_bytes, stream);
-    run->launches += 1;
+    if (e == cudaSuccess) run->launches += 1;
+    else cudaGetLastError();  // returned here, not left pending for a later call
     return e;
 }
 
