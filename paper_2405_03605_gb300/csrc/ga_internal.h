@@ -63,7 +63,8 @@ inline cudaError_t pool_free(void *p, cudaStream_t stream) { return cudaFreeAsyn
 // another starts at multiples of 2.06 us on this GPU.  One launch per generation, ordinary and
 // dependent: 131,000 agents 6.2 and 3.9 us, 1.3M 10.3 and 8.9, 4.2M 27.0 and 25.0, 16.8M 92.6
 // and 89.9; 4.2M agents of 48 bytes 72.3 and 69.7.  (Releasing the next grid at the start of each,
-// so that its blocks wait on the SMs, is slower: 13.2 and 90.8 us for 1.3M and 16.8M.)
+// so that its blocks wait on the SMs, is slower: 13.2 and 90.8 us for 1.3M and 16.8M.)  A failed
+// launch's error is returned and not left pending, where a later call would take it for its own.
 template <typename... P, typename... A>
 cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream,
                              A... args)
@@ -78,7 +79,9 @@ cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, cudaSt
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 // Workspace header: the device status word (first 256 bytes), then the curation-site table
