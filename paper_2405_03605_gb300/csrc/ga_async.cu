@@ -191,7 +191,7 @@ island_async_kernel(const AsyncArgs a)
         const size_t agent = static_cast<size_t>(island) * N + seg_lane + 32u * ag;
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
-            const uint4 v = __ldg(&p.src[agent * Q + q]);
+            const uint4 v = p.src[agent * Q + q];
             const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e)
@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(kAsyncThreads) island_async_gen_kernel(const A
     if (valid) {
 #pragma unroll
         for (int ag = 0; ag < A; ++ag) {
-            const uint4 v = __ldg(&p.src[static_cast<size_t>(island) * N + seg_lane + 32u * ag]);
+            const uint4 v = p.src[static_cast<size_t>(island) * N + seg_lane + 32u * ag];
             rec[ag][0] = v.x;
             rec[ag][1] = v.y;
             rec[ag][2] = v.z;

@@ -29,9 +29,12 @@
 
 namespace ga {
 
-// Everything one launch needs to know about one run.
+// Everything one launch needs to know about one run.  What earlier launches of the stream write
+// (records, site table, masks) is read with plain loads: a dependent launch may be in flight while
+// they are still being written, so they are not constant for the kernel's lifetime, as __ldg and a
+// const __restrict__ pointer would promise, and such loads could move over the wait.
 struct RunParams {
-    const uint4 *__restrict__ src;          // records before generation g0
+    const uint4 *src;                       // records before generation g0
     uint4 *__restrict__ dst;                // records after generation g0 + n_gens - 1
     uint32_t rows, cols, n_islands;
     uint32_t cols_m, cols_l;                // island / cols as a multiply-shift (div_cols)
@@ -40,14 +43,14 @@ struct RunParams {
     uint32_t policy, log2_sites, sites, bits;
     uint32_t run_id;
     uint32_t g0, n_gens, migrate;           // migration (if set) happens at g0 only
-    const int32_t *__restrict__ gen_sites;  // curation site of generation g0 + i
+    const int32_t *gen_sites;               // curation site of generation g0 + i
     float effect_scale;                     // fitness model: mutation amount scale
     uint32_t gen_sites_left;                // entries of gen_sites from g0 on
     int *status;                            // the run's device status word
     // deposit masks of generation g0 + i (records with a 64-bit surface, S b <= 64): the bits of
     // surface words 0 and 1 that the generation's deposit overwrites, (0, 0) for none; the
     // differentia (low b bits of the draw) is spread over every b-bit field by one multiply
-    const uint2 *__restrict__ gen_masks;
+    const uint2 *gen_masks;
     uint32_t dif_mask, dif_rep;             // 2^b - 1 and the b-bit repetition pattern
 };
 
@@ -55,14 +58,14 @@ struct RunParams {
 // device-check build finds `it` past the table).
 __device__ __forceinline__ int gen_site_at(const RunParams &p, uint32_t it)
 {
-    return in_bounds(it < p.gen_sites_left, p.status) ? __ldg(&p.gen_sites[it]) : -1;
+    return in_bounds(it < p.gen_sites_left, p.status) ? p.gen_sites[it] : -1;
 }
 
 // Deposit masks of generation g0 + it ((0, 0), no deposit, if a device-check build finds `it`
 // past the table).
 __device__ __forceinline__ uint2 gen_mask_at(const RunParams &p, uint32_t it)
 {
-    return in_bounds(it < p.gen_sites_left, p.status) ? __ldg(&p.gen_masks[it]) : make_uint2(0u, 0u);
+    return in_bounds(it < p.gen_sites_left, p.status) ? p.gen_masks[it] : make_uint2(0u, 0u);
 }
 
 // Candidate trait of slot `sel` of this lane's island.  For N <= 32 `sel` may carry extra
@@ -183,7 +186,8 @@ static __device__ __noinline__ int curation_site_of(uint32_t policy, uint32_t lo
 // MODEL 0: int32 trait, +1 / -1; MODEL 1: float fitness, -/+ effect_scale * |normal|.
 // DM = 1 (64-bit surfaces, every counter equal to g): the deposit takes the generation's
 // precomputed masks `dmask` instead of the site: the differentia spread over every b-bit
-// field, kept where the mask is set -- the same bits as writing it at site * b.
+// field, kept where the mask is set -- the same bits as writing it at site * b.  DM = 2: as 1, the
+// masks read where they are needed, gen_site being the generation's index in the launch.
 // PRE = 1 (float model): the births' signed mutation amounts come in `amount`, used where `mutates`,
 // instead of being drawn here.
 template <int N, int SW, int TS, int MODEL, int CF = 1, int DM = 0, int PRE = 0>
@@ -341,6 +345,8 @@ __device__ __forceinline__ void reproduce(uint32_t (&rec)[Shape<N>::A][2 + SW],
         }
         if constexpr (DM != 0) {
             static_assert(SW == 2 && CF == 0, "mask deposits: 64-bit surfaces, uniform counters");
+            if constexpr (DM == 2)
+                if (ag == 0) dmask = gen_mask_at(p, static_cast<uint32_t>(gen_site));
             const uint32_t rep = (w[ag].w & p.dif_mask) * p.dif_rep;
             child[ag][2] = (child[ag][2] & ~dmask.x) | (rep & dmask.x);
             child[ag][3] = (child[ag][3] & ~dmask.y) | (rep & dmask.y);
@@ -447,7 +453,7 @@ __device__ __forceinline__ void step_block(const RunParams &p, const RoundKeys &
             const uint4 *srec = p.src + (static_cast<size_t>(nb) * N + e) * Q;
             if (in_bounds(nb < p.n_islands && e < static_cast<uint32_t>(N), p.status)) {
 #pragma unroll
-                for (int q = 0; q < Q; ++q) imm[q] = __ldg(&srec[q]);
+                for (int q = 0; q < Q; ++q) imm[q] = srec[q];
             } else {
 #pragma unroll
                 for (int q = 0; q < Q; ++q) imm[q] = make_uint4(0u, 0u, 0u, 0u);
@@ -464,7 +470,7 @@ __device__ __forceinline__ void step_block(const RunParams &p, const RoundKeys &
             const size_t agent = static_cast<size_t>(island) * N + seg_lane + 32u * ag;
 #pragma unroll
             for (int q = 0; q < Q; ++q) {
-                const uint4 v = __ldg(&p.src[agent * Q + q]);
+                const uint4 v = p.src[agent * Q + q];
                 const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
@@ -747,6 +753,11 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
     };
 
     const uint2 dmask = gen_mask_at(p, 0u);
+    // islands of 64: the mask of a later generation read only where it is needed, as it would occupy
+    // registers that the shared lookups want (16 generations to a launch, 500,000 agents 3.24 us per
+    // generation, 3.38 read before; smaller islands up to 5% slower so)
+    constexpr int kLaterMasks = N >= 64 ? 2 : 1;
+    auto later_mask = [&](uint32_t it) { return kLaterMasks == 2 ? make_uint2(0u, 0u) : gen_mask_at(p, it); };
     const SlotDraws<N> sd = slot_draws<N>(p, rk, p.g0, seg_lane);
     // UNROLL: fully unrolled over the block's units, so the double-buffer index, the
     // shared-memory offsets of each unit and the loop control become constants (94.2 against
@@ -858,8 +869,8 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
                     Lookup traits;
                     if constexpr (kShared) traits.traits = reinterpret_cast<int *>(&s_kept[warp][h * A][0]) + (it & 1u) * N;
                     birth_draws<N>(w, p, rk, p.g0 + it, island, seg_lane);
-                    reproduce<N, SW, TS, 1, 0, 1>(rec, w, p, rk, island, seg_lane, mask, p.g0 + it, 0,
-                                                  gen_mask_at(p, it), nullptr, nullptr, traits);
+                    reproduce<N, SW, TS, 1, 0, kLaterMasks>(rec, w, p, rk, island, seg_lane, mask, p.g0 + it, it,
+                                                            later_mask(it), nullptr, nullptr, traits);
                 }
                 uint4 *dst = p.dst + static_cast<size_t>(first) * N + lane;
 #pragma unroll
@@ -910,8 +921,8 @@ __device__ __forceinline__ void step_units(const RunParams &p, const RoundKeys &
         reproduce<N, SW, TS, MODEL, 0, 1>(rec, w, p, rk, island, seg_lane, mask, p.g0, 0, dmask);
         for (uint32_t it = 1; !ONE && it < p.n_gens; ++it) {
             birth_draws<N>(w, p, rk, p.g0 + it, island, seg_lane);
-            reproduce<N, SW, TS, MODEL, 0, 1>(rec, w, p, rk, island, seg_lane, mask, p.g0 + it, 0,
-                                              gen_mask_at(p, it), nullptr, nullptr, lookup());
+            reproduce<N, SW, TS, MODEL, 0, kLaterMasks>(rec, w, p, rk, island, seg_lane, mask, p.g0 + it, it,
+                                                        later_mask(it), nullptr, nullptr, lookup());
         }
         uint4 *dst = p.dst + static_cast<size_t>(first) * N + lane;
 #pragma unroll

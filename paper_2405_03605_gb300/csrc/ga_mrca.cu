@@ -3,7 +3,9 @@
 //
 // Synchronous runs (one counter T) take two launches, pack_kernel and pair_kernel; asynchronous
 // ones (counters differ) two others, mixed_table_kernel and mixed_pair_kernel (each described
-// there).
+// there).  The second kernel of each pair is in flight while the first still writes what it reads, and
+// the first may be while an earlier launch writes the population: inputs are read with plain loads
+// behind the wait, not as constant data (__ldg, const __restrict__), which a compiler may move.
 #include "ga_device.cuh"
 #include "ga_internal.h"
 
@@ -198,19 +200,19 @@ __device__ __forceinline__ uint32_t pair_entry(const String8 &a, const String8 &
 // The string of sampled agent a of n: W = 2, an 8-byte word each; W = 8, two arrays of 16 bytes.
 __device__ __forceinline__ void read_string(const void *packed, uint32_t, uint32_t a, uint2 &v)
 {
-    v = __ldg(static_cast<const uint2 *>(packed) + a);
+    v = static_cast<const uint2 *>(packed)[a];
 }
 __device__ __forceinline__ void read_string(const void *packed, uint32_t n, uint32_t a, String8 &v)
 {
-    v.h[0] = __ldg(static_cast<const uint4 *>(packed) + a);
-    v.h[1] = __ldg(static_cast<const uint4 *>(packed) + n + a);
+    v.h[0] = static_cast<const uint4 *>(packed)[a];
+    v.h[1] = static_cast<const uint4 *>(packed)[n + a];
 }
 
 // W: words of a string (2: S b <= 64; 8: up to 256 bits).
 template <uint32_t W>
 __global__ void __launch_bounds__(256)
-pack_kernel(const uint4 *__restrict__ pop, uint32_t record_quads, uint32_t n_agents,
-            const uint32_t *__restrict__ ids, uint32_t n, uint32_t policy, uint32_t log2_sites,
+pack_kernel(const uint4 *pop, uint32_t record_quads, uint32_t n_agents,
+            const uint32_t *ids, uint32_t n, uint32_t policy, uint32_t log2_sites,
             uint32_t log2_bits, uint32_t K, uint32_t T, uint2 *__restrict__ tab,
             void *__restrict__ packed, int *__restrict__ status)
 {
@@ -250,22 +252,22 @@ pack_kernel(const uint4 *__restrict__ pop, uint32_t record_quads, uint32_t n_age
 #pragma unroll
     for (uint32_t e = 0; e < W; ++e) w[e] = 0u;
     if (a < n) {
-        const uint32_t id = __ldg(&ids[a]);
+        const uint32_t id = ids[a];
         if (id >= n_agents) {
             atomicCAS(status, GA_OK, GA_EINVAL);
         } else {
             const uint4 *r = pop + static_cast<size_t>(id) * record_quads;
-            const uint4 q0 = __ldg(&r[0]);
+            const uint4 q0 = r[0];
             w[0] = q0.z;
             w[1] = words > 1u ? q0.w : 0u;
             if constexpr (W > 2u) {  // records of 32 or 48 bytes
-                const uint4 q1 = __ldg(&r[1]);
+                const uint4 q1 = r[1];
                 w[2] = q1.x;
                 w[3] = words > 3u ? q1.y : 0u;
                 w[4] = words > 4u ? q1.z : 0u;
                 w[5] = words > 5u ? q1.w : 0u;
                 if (record_quads > 2u) {
-                    const uint4 q2 = __ldg(&r[2]);
+                    const uint4 q2 = r[2];
                     w[6] = words > 6u ? q2.x : 0u;
                     w[7] = words > 7u ? q2.y : 0u;
                 }
@@ -318,7 +320,7 @@ __device__ __forceinline__ void first_pair(uint32_t n, uint32_t p, uint32_t &i, 
 
 template <uint32_t W>
 __global__ void __launch_bounds__(kPairThreads)
-pair_kernel(const void *__restrict__ packed, uint32_t n, const uint2 *__restrict__ tab_g,
+pair_kernel(const void *packed, uint32_t n, const uint2 *tab_g,
             uint32_t per_warp, uint32_t *__restrict__ lo, uint32_t *__restrict__ hi, int *__restrict__ status)
 {
     __shared__ uint2 tab[32 * W + 1];
@@ -440,8 +442,8 @@ size_t carve_mixed(void *scratch, uint32_t S, uint32_t bits, uint32_t n, MixedLa
 // agent's counter and puts it at its site, then sorts site k among the occupied ones by
 // counting the smaller ranks.
 __global__ void __launch_bounds__(256)
-mixed_table_kernel(const uint32_t *__restrict__ pop, uint32_t record_words, uint32_t n_agents,
-                   const uint32_t *__restrict__ ids, uint32_t n, uint32_t policy,
+mixed_table_kernel(const uint32_t *pop, uint32_t record_words, uint32_t n_agents,
+                   const uint32_t *ids, uint32_t n, uint32_t policy,
                    uint32_t log2_sites, uint32_t words, uint32_t *__restrict__ cnt,
                    uint32_t *__restrict__ held, uint32_t *__restrict__ surf,
                    uint32_t *__restrict__ ranks, uint8_t *__restrict__ order,
@@ -489,9 +491,9 @@ mixed_table_kernel(const uint32_t *__restrict__ pop, uint32_t record_words, uint
 template <uint32_t THREADS, bool BIT>
 __global__ void __launch_bounds__(THREADS)
 mixed_pair_kernel(uint32_t n, uint32_t sites, uint32_t words, uint32_t bits, uint32_t K,
-                  const uint32_t *__restrict__ cnt, const uint32_t *__restrict__ held,
-                  const uint32_t *__restrict__ surf, const uint32_t *__restrict__ ranks,
-                  const uint8_t *__restrict__ order, uint32_t *__restrict__ lo,
+                  const uint32_t *cnt, const uint32_t *held,
+                  const uint32_t *surf, const uint32_t *ranks,
+                  const uint8_t *order, uint32_t *__restrict__ lo,
                   uint32_t *__restrict__ hi, int *__restrict__ status)
 {
     constexpr uint32_t kNone = 0xFFFFFFFFu;
@@ -510,13 +512,13 @@ mixed_pair_kernel(uint32_t n, uint32_t sites, uint32_t words, uint32_t bits, uin
     for (uint32_t t = warp; t < 3u * words; t += THREADS / 32u) {
         const uint32_t g = t / words, w = t - g * words;
         const uint32_t a = first_of(g) + lane;
-        const uint32_t v = a < n ? __ldg(&surf[static_cast<size_t>(a) * words + w]) : 0u;
+        const uint32_t v = a < n ? surf[static_cast<size_t>(a) * words + w] : 0u;
         plane[g][32u * w + lane] = transpose(v);
     }
     if (threadIdx.x < 96u) {
         const uint32_t g = threadIdx.x >> 5, a = first_of(g) + lane;
-        count[g][lane] = a < n ? __ldg(&cnt[a]) : 0u;
-        held_s[g][lane] = a < n ? __ldg(&held[a]) : 0u;
+        count[g][lane] = a < n ? cnt[a] : 0u;
+        held_s[g][lane] = a < n ? held[a] : 0u;
     }
     __syncthreads();
 
@@ -541,7 +543,7 @@ mixed_pair_kernel(uint32_t n, uint32_t sites, uint32_t words, uint32_t bits, uin
 #pragma unroll
             for (int g = 0; g < NG; ++g) differ[g] = 0u;
             if (c0 + lane < m) {
-                const uint32_t q0 = (c0 == 0u ? site0 : __ldg(&od[c0 + lane])) * (BIT ? 1u : bits);
+                const uint32_t q0 = (c0 == 0u ? site0 : od[c0 + lane]) * (BIT ? 1u : bits);
                 if (in_bounds(q0 + bits <= 32u * words, status)) {
                     for (uint32_t q = q0; q < q0 + (BIT ? 1u : bits); ++q) {
                         const uint32_t mine = 0u - ((plane[gb][q] >> bl) & 1u);
@@ -566,25 +568,25 @@ mixed_pair_kernel(uint32_t n, uint32_t sites, uint32_t words, uint32_t bits, uin
         for (int g = 0; g < NG; ++g) {
             if (!active[g]) continue;
             // a mismatch at a rank not below Ta lies past the common prefix
-            const uint32_t fr = first[g] != kNone ? __ldg(&rk[first[g]]) : kNone;
-            const uint32_t fl = first[g] != kNone && first[g] >= K ? __ldg(&rk[first[g] - K]) + 1u : 0u;
+            const uint32_t fr = first[g] != kNone ? rk[first[g]] : kNone;
+            const uint32_t fl = first[g] != kNone && first[g] >= K ? rk[first[g] - K] + 1u : 0u;
             h[g] = fr;
             l[g] = fl;
             if (fr >= Ta[g]) {  // no common rank differs: the prefix ends at the first rank >= Ta
                 uint32_t below = 0, above = m;
                 while (below < above) {
                     const uint32_t mid = (below + above) >> 1;
-                    if (__ldg(&rk[mid]) < Ta[g]) below = mid + 1u;
+                    if (rk[mid] < Ta[g]) below = mid + 1u;
                     else above = mid;
                 }
                 h[g] = Ta[g];
-                l[g] = below >= K ? __ldg(&rk[below - K]) + 1u : 0u;
+                l[g] = below >= K ? rk[below - K] + 1u : 0u;
             }
         }
     };
     // the site at rank index `lane` of sampled agent a (0 where there is none)
     auto first_site = [&](uint32_t a) {
-        return a < n && lane < sites ? static_cast<uint32_t>(__ldg(&order[static_cast<size_t>(a) * sites + lane])) : 0u;
+        return a < n && lane < sites ? static_cast<uint32_t>(order[static_cast<size_t>(a) * sites + lane]) : 0u;
     };
 
     // pairs whose row agent holds the larger counter (or the same): b = row, lanes = columns

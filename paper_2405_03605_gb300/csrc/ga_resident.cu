@@ -136,6 +136,13 @@ __device__ __forceinline__ uint32_t load_relaxed(const uint32_t *p)
     return v;
 }
 
+// Deposit masks of the launch's generation `it` ((0, 0) past the table in a device-check build).  The
+// resident kernel starts when the set-up kernel that wrote them has ended, so they are constant.
+__device__ __forceinline__ uint2 const_mask_at(const RunParams &p, uint32_t it)
+{
+    return in_bounds(it < p.gen_sites_left, p.status) ? __ldg(&p.gen_masks[it]) : make_uint2(0u, 0u);
+}
+
 // Next migration generation at or after g (~0u: none before `end`).
 __device__ __forceinline__ uint32_t next_migration(uint32_t g, uint32_t end, uint32_t k, uint32_t on)
 {
@@ -251,7 +258,7 @@ __global__ void __launch_bounds__(32, WARPS) resident_kernel(const ResidentArgs 
         const uint32_t g = p.g0 + it;
         uint2 dm = make_uint2(0u, 0u);
         int site = -1;
-        if constexpr (SW == 2) dm = gen_mask_at(p, it);
+        if constexpr (SW == 2) dm = const_mask_at(p, it);
         else site = gen_site_at(p, it);
         const SlotDraws<N> sd = slot_draws<N>(p, a.rk, g, seg_lane);
         uint4 w[A];
@@ -377,7 +384,7 @@ __global__ void __launch_bounds__(32, WARPS) resident_kernel(const ResidentArgs 
                 reproduce<N, SW, TS, MODEL, 0, 1>(rec, w, p, a.rk, island, seg_lane, mask, g, 0, dm);
                 if constexpr (IV) {
                     for (uint32_t j = 1; j < len; ++j) {
-                        const uint2 dj = gen_mask_at(p, it + j);
+                        const uint2 dj = const_mask_at(p, it + j);
                         birth_draws<N>(w, p, a.rk, g + j, island, seg_lane);
                         reproduce<N, SW, TS, MODEL, 0, 1>(rec, w, p, a.rk, island, seg_lane, mask, g + j, 0, dj);
                     }

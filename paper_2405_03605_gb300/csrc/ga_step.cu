@@ -21,9 +21,14 @@ constexpr int step_warps() { return N <= 8 && SW <= 2 ? 8 : 4; }
 
 // Blocks per SM asked of the compiler: 12 (40 registers) for 48-byte records with equal counters
 // in islands of 16 and 32, which take 44 to 46 unasked: 61.7 against 63.9 us a generation for 4.2M
-// agents in islands of 32, 15.5 against 15.9 for 1M.
+// agents in islands of 32, 15.5 against 15.9 for 1M.  7 (64 to 68 registers) for 16-byte records with equal
+// counters in islands of 128, which take 80 unasked: 500,000 agents 4.4 against 5.2 us with a migration
+// every generation, 2.14 against 2.18 every 16.
 template <int N, int SW, int CF>
-constexpr int step_min_blocks() { return SW == 8 && CF == 0 && (N == 16 || N == 32) ? 12 : 1; }
+constexpr int step_min_blocks()
+{
+    return CF != 0 ? 1 : SW == 8 && (N == 16 || N == 32) ? 12 : SW == 2 && N == 128 ? 7 : 1;
+}
 
 // Single run: per-run values and round keys are kernel parameters (constant bank).
 struct StepArgs {
