@@ -184,10 +184,13 @@ int ga_async_window(ga_run *run, uint32_t window);
  * the generation, at most 8,192 islands, of which at most 40 of 32 agents and 32 of 64 agents
  * for each SM of the device; the mailboxes (128 bytes per island) are part of the workspace of
  * such runs.  Other runs keep theirs in the population buffer that the launch writes at its end.
- * wait_limit_us bounds every wait for a mailbox (wall clock, default 1,000,000 = 1 s): when
- * it runs out the launch records GA_ETIMEOUT, every warp leaves at its next migration
- * generation, the population is undefined, and the next ga_sync returns GA_ETIMEOUT (the
- * run can then be reset or loaded and stepped again).  Errors: GA_EINVAL (mode, limit 0).
+ * wait_limit_us bounds every wait for a mailbox (wall clock, default 1,000,000 = 1 s; at least
+ * 4,096 reads of the mailbox, some milliseconds, are made first, so that time in which the GPU ran
+ * other work does not end a wait): when it runs out the launch records GA_ETIMEOUT, every warp
+ * leaves at its next migration generation, the population is undefined, and the next ga_sync
+ * returns GA_ETIMEOUT (the run can then be reset or loaded and stepped again).  That holds for
+ * every run that GA_RESIDENT_AUTO steps resident; GA_RESIDENT_OFF has no waits.
+ * Errors: GA_EINVAL (mode, limit 0).
  */
 #define GA_RESIDENT_AUTO 0u
 #define GA_RESIDENT_OFF 1u

@@ -32,8 +32,8 @@
 // each island's in the place of its own records: those are written when the launch ends, by
 // the warp that has read the island's last arrival.
 //
-// Waits are bounded: a poll gives up after the run's wait limit (wall clock, %globaltimer),
-// records GA_ETIMEOUT in the status word and sets the launch's abort word; every poll also
+// Waits are bounded: a poll gives up after the run's wait limit (wall clock, %globaltimer) and
+// kMinPolls reads, records GA_ETIMEOUT in the status word and sets the launch's abort word; every poll also
 // watches the abort word, so once one warp gives up every warp leaves at its next migration
 // generation.  The population is then undefined; the status is returned by the next ga_sync.
 //
@@ -83,6 +83,11 @@ uint32_t units_per_warp(const ga_run *run, uint32_t n_units, uint32_t sms)
     const uint32_t units = (n_units + 18u * sms - 1u) / (18u * sms);
     return units < 2u ? 2u : units;
 }
+
+// Reads that a wait makes at least before it gives up (3 to 5 ms).  The clock goes on while the GPU runs
+// another process; without them a launch that was set aside for longer than the limit would give up
+// though its neighbours are about to answer.
+constexpr uint32_t kMinPolls = 4096;
 
 struct ResidentArgs {
     RunParams r;
@@ -320,7 +325,7 @@ __global__ void __launch_bounds__(32, WARPS) resident_kernel(const ResidentArgs 
                             gave_up = true;
                             break;
                         }
-                        if (global_ns() - t0 > a.wait_ns) {
+                        if (global_ns() - t0 > a.wait_ns && polls >= kMinPolls) {
                             atomicCAS(p.status, 0, GA_ETIMEOUT);
                             atomicExch(a.abort_word, 1u);
                             gave_up = true;
