@@ -88,6 +88,10 @@ def shapes(args, rank):
     return out
 
 
+def parallelism(world):
+    return f"replicas x{world}" if world > 1 else "1 GPU"
+
+
 def workload_config(args, sh):
     return {
         "workload": (f"island GA {args.rows}x{args.cols} torus x {sh.island_size} agents "
@@ -172,7 +176,7 @@ ISLAND_STEP_TRAFFIC = {"kernel": "island_units_kernel<32,5,0,true>", "bytes": 44
                        "rows": 512, "cols": 1024, "island_size": 32}
 # warp-instructions per island-generation of the resident kernel on the 32x32 torus
 # (smsp__inst_executed.sum of a 200-generation launch / (1,024 islands x 200), this build)
-RESIDENT_INST = {"kernel": "resident_kernel<32,2,5,0,0>", "inst_per_island_gen": 77725590 / 204800}
+RESIDENT_INST = {"kernel": "resident_kernel<32,2,5,0,0,20>", "inst_per_island_gen": 77670310 / 204800}
 
 
 def aggregate_replicas(elapsed_ms, agent_gens, world, device="cpu"):
@@ -248,7 +252,7 @@ def run_reference(args, rank, world):
         "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": dt * 1000 / args.steps, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "u32", "data": "synthetic",
-        "config": workload_config(args, sh),
+        "config": {**workload_config(args, sh), "parallelism": parallelism(world)},
         "cpu_baseline": {"value": value, "unit": UNIT, "cores": threads, "kind": "oracle",
                          "sample": sample},
         "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 0,
@@ -278,8 +282,7 @@ def run_ours(args, rank, world, local):
     line = {"metric": METRIC, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "u32", "data": "synthetic",
-            "config": {**workload_config(args, shs[0]),
-                       "parallelism": f"replicas x{world}" if world > 1 else "1 GPU"}}
+            "config": {**workload_config(args, shs[0]), "parallelism": parallelism(world)}}
     launches = 0
     clk = None
     if args.run["main"]:
@@ -595,7 +598,8 @@ def measure_variants(args):
     hybrid), islands of 16/32/64, migration every 1/4/16 generations: agent-generations/s
     from founder populations, CUDA events on the run's stream, with the algorithmic HBM
     bytes per agent-generation (record in and out once per launch plus the immigrant
-    records, 2G/k + 4G/(N k)) turned into a fraction of the measured copy bandwidth."""
+    records, 2G/k + 4G/(N k)) turned into a fraction of the measured copy bandwidth (above 1
+    where the immigrants' reads hit L2), and the same without the immigrants."""
     import torch
     from paper_2405_03605_gb300 import ga
     from paper_2405_03605_gb300.workloads import variant_shapes
@@ -622,7 +626,8 @@ def measure_variants(args):
                 b_alg = 2 * G / k + 4 * G / (n * k)
                 out.append({"variant": name, "island_size": n, "migrate_every": k,
                             "record_bytes": G, "agent_gens_per_s": rate,
-                            "hbm_frac": rate * b_alg / 1e9 / peak})
+                            "hbm_frac": rate * b_alg / 1e9 / peak,
+                            "hbm_frac_records": rate * 2 * G / k / 1e9 / peak})
                 r.close()
     return {"agents": 4194304, "generations": gens, "runs": out}
 
