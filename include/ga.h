@@ -182,7 +182,7 @@ int ga_async_window(ga_run *run, uint32_t window);
  *   GA_RESIDENT_ON    resident launches; ga_step returns GA_EUNSUPPORTED if not eligible.
  * Eligible for GA_RESIDENT_ON: GA_SYNC, 16-byte records, island sizes 8 to 64, counters equal to
  * the generation, at most 8,192 islands, of which at most 40 of 32 agents and 32 of 64 agents
- * for each SM of the device; the mailboxes (128 bytes per island) are part of the workspace of
+ * (36 of 64 for the trait model with tournaments of 5) for each SM of the device; the mailboxes (128 bytes per island) are part of the workspace of
  * such runs.  Other runs keep theirs in the population buffer that the launch writes at its end.
  * wait_limit_us bounds every wait for a mailbox (wall clock, default 1,000,000 = 1 s; at least
  * 4,096 reads of the mailbox, some milliseconds, are made first, so that time in which the GPU ran

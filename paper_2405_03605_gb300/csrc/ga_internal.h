@@ -57,14 +57,15 @@ cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t stream);
 inline cudaError_t pool_free(void *p, cudaStream_t stream) { return cudaFreeAsync(p, stream); }
 
 // Launch `kernel` as a programmatic dependent of the previous kernel on `stream` (see
-// wait_previous_grid in ga_device.cuh).  Every kernel of a chain of launches goes this way, with
-// the wait as its first instruction and no early release: nothing overlaps, but the launch is
-// handed over as soon as the previous grid's blocks have left, where an ordinary launch after
-// another starts at multiples of 2.06 us on this GPU.  One launch per generation, ordinary and
-// dependent: 131,000 agents 6.2 and 3.9 us, 1.3M 10.3 and 8.9, 4.2M 27.0 and 25.0, 16.8M 92.6
-// and 89.9; 4.2M agents of 48 bytes 72.3 and 69.7.  (Releasing the next grid at the start of each,
-// so that its blocks wait on the SMs, is slower: 13.2 and 90.8 us for 1.3M and 16.8M.)  A failed
-// launch's error is returned and not left pending, where a later call would take it for its own.
+// wait_previous_grid in ga_device.cuh).  The launches of a single run go this way (a batch's class
+// launches and the cooperative ones are ordinary), the steps' with the wait as their first
+// instruction and no early release: nothing overlaps, but the launch is handed over as soon as the
+// previous grid's blocks have left, where an ordinary launch after another starts at multiples of
+// 2.06 us on this GPU.  One launch per generation, ordinary and dependent: 131,000 agents 6.2 and
+// 3.9 us, 1.3M 10.3 and 8.9, 4.2M 27.0 and 25.0, 16.8M 92.6 and 89.9; 4.2M agents of 48 bytes 72.3
+// and 69.7.  (Releasing the next grid at the start of each, so that its blocks wait on the SMs, is
+// slower: 13.2 and 90.8 us for 1.3M and 16.8M.)  A failed launch's error is returned and not left
+// pending, where a later call would take it for its own.
 template <typename... P, typename... A>
 cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream,
                              A... args)

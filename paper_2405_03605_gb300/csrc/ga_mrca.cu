@@ -402,7 +402,7 @@ cudaError_t launch_sync_mrca(const void *pop, uint32_t record_bytes, uint32_t n_
 //                      agent), so lane l looks up the mismatches of all 32 agents at b's l-th
 //                      rank in one word, and a 32 x 32 bit transpose hands every lane its own
 //                      agent's mismatches in b's rank order: the first set bit is the answer.
-// Issue-bound: some 200 warp-instructions per 32 pairs, against 2,757 for one thread per pair
+// Issue-bound: 215 warp-instructions per 32 pairs (the tables 25 more), against 2,757 for one thread per pair
 // walking both agents' sites twice.  The whole call for 3,001 agents with 64 sites (4.5M pairs, 36
 // MB of bounds): 47 us, 376 us before; 2,816 agents with 256 sites 122 us, 1,371 before.
 // ---------------------------------------------------------------------------------------

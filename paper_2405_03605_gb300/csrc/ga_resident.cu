@@ -3,8 +3,8 @@
 // trade migrants through mailboxes in global memory (L2) instead of through launch boundaries.
 // The paper's processors keep their populations in place and exchange only migrants with their
 // neighbours (Sec. 2); this is that arrangement on the GPU.  A launch per generation cannot
-// follow it there: launches on one stream start at least 4 us apart, and a run of 320,000
-// agents needs 2 us of arithmetic per generation.
+// follow it there: it takes at least 2.4 us, even as a dependent one, and 4.3 for a run of 320,000
+// agents, whose arithmetic needs 2.
 //
 // Scope: synchronous runs whose counters all equal the generation, any record size, islands of
 // 8 to 64 agents.  Results are bit-identical to the streamed kernels: the same draws, landing
@@ -518,7 +518,8 @@ __global__ void resident_init_kernel(uint4 *__restrict__ mail, uint32_t n_island
 size_t resident_state_bytes(uint32_t n_islands, uint32_t record_bytes)
 {
     if (record_bytes != 16u || n_islands > kResidentMaxIslands) return 0;
-    // 256 bytes, then two parities of four 16-byte mailboxes per island
+    // 256 bytes that nothing uses (callers may have sized workspaces by them), then two parities of four
+    // 16-byte mailboxes per island
     return 256u + static_cast<size_t>(n_islands) * 4u * 2u * 16u;
 }
 
