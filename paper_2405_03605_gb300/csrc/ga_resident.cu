@@ -172,11 +172,27 @@ __host__ __device__ constexpr uint32_t warp_bytes(uint32_t islands)
     return islands * (N * Record<SW>::Q * 16u + 4u * (4u + 2u + 1u) + 4u);
 }
 
+// Resident warps per SM asked of the compiler, for the registers that leaves (20: 96, 28: 72, 32: 64).
+// Fewer registers let the warps of runs on other streams fit beside this one's, and few of them hold a
+// single run back: 16-byte records in islands of 32 take 74 to 78 unasked and 62 to 64 here without a
+// spill.  65,536 agents, us per generation for one run and for four at once: 1.48 and 6.2 with 20, 1.40
+// and 4.0 with 32 (before islands shared warps 1.61 and 4.0); float model 1.98 and 8.3, 1.88 and 5.8.  20
+// where the cap costs a single run more than 5% for some size: float runs in islands of 64, and of 16
+// with several generations to a migration, and tournaments of 5 in islands of 64 with several; wider
+// records, which were not slower beside one another.
+template <int N, int SW, int TS, int MODEL, bool IV>
+constexpr int resident_warps()
+{
+    if (SW != 2) return 20;
+    if (N == 64) return MODEL == 0 && (!IV || TS == 0) ? 28 : 20;
+    if (N == 32) return MODEL == 1 && IV ? 28 : 32;
+    if (N == 16) return !IV ? 32 : MODEL == 0 ? 28 : 20;
+    return 28;
+}
+
 // N, SW, TS, MODEL: island size, surface words, tournament size (0: read from the run) and genome
-// model, as in step_block; IV: migrations more than a generation apart.  WARPS: resident warps per SM
-// asked of the compiler: 20 (96 registers), or 28 (72, a few spilled) for float runs in islands of 16
-// that need them (see pick_ts; 40,000 agents do not: 1.09 against 1.05 us every 4 generations).
-template <int N, int SW, int TS, int MODEL, bool IV, int WARPS = 20>
+// model, as in step_block; IV: migrations more than a generation apart.
+template <int N, int SW, int TS, int MODEL, bool IV, int WARPS = resident_warps<N, SW, TS, MODEL, IV>()>
 __global__ void __launch_bounds__(32, WARPS) resident_kernel(const ResidentArgs a)
 {
     constexpr int A = Shape<N>::A, P = Shape<N>::P, SEG = Shape<N>::SEG;
