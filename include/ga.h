@@ -177,7 +177,9 @@ int ga_async_window(ga_run *run, uint32_t window);
  *                     to the generation, island sizes 8 to 64, a population that the device
  *                     holds at once, and migrations frequent enough for its size (every
  *                     generation: up to a million agents in islands of 32, 1.4 million of 64);
- *                     streamed launches otherwise, and where a resident one is refused
+ *                     streamed launches otherwise, where a resident one is refused, and for
+ *                     large runs of 16-byte records while another large run steps resident on
+ *                     another stream
  *   GA_RESIDENT_OFF   one launch per migration interval, the population streamed;
  *   GA_RESIDENT_ON    resident launches; ga_step returns GA_EUNSUPPORTED if not eligible.
  * Eligible for GA_RESIDENT_ON: GA_SYNC, 16-byte records, island sizes 8 to 64, counters equal to

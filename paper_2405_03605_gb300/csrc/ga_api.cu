@@ -142,18 +142,102 @@ cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t stream)
     return cudaMallocFromPoolAsync(p, bytes, pool, stream);
 }
 
+// Resident launches of runs that only GA_RESIDENT_AUTO steps so (large ones) fill the GPU, and several
+// on different streams take turns, where streamed launches fill one another's gaps: 320,000 agents, us
+// per generation of two, four and eight runs at once, resident in turn 5.3, 11.0 and 22.6, streamed
+// 6.0, 8.5 and 14.3.  So a run of 16-byte records streams while another such launch is in flight on
+// another stream of its device: 6.9, 8.8 and 13.5 (9.0, 12.1 and 17.7 before such runs stepped
+// resident; letting two or three in turn is slower from three runs on).  Wide records are faster
+// resident however many runs there are (eight of 320,000 agents 25.8 against 42.2).  What is in flight
+// is asked of an event behind each such launch; a stream that is being captured neither asks nor
+// records.
+namespace {
+
+std::mutex in_flight_mu;
+ga_run *in_flight = nullptr;  // runs with an event that was not complete when last asked
+
+// Event calls that must not disturb a capture of another thread.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+bool capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
+bool another_resident(const ga_run *run, cudaStream_t stream)
+{
+    int dev = 0;
+    if (capturing(stream) || cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lock(in_flight_mu);
+    const RelaxedCapture relaxed;
+    for (ga_run **at = &in_flight; *at;) {
+        ga_run *r = *at;
+        if (r == run || r->resident_stream == stream || r->resident_device != dev) {
+            at = &r->resident_next;
+            continue;
+        }
+        const cudaError_t e = cudaEventQuery(r->resident_done);
+        if (e != cudaSuccess) cudaGetLastError();
+        if (e == cudaErrorNotReady) return true;
+        r->resident_listed = false;
+        *at = r->resident_next;
+    }
+    return false;
+}
+
+void note_resident(ga_run *run, cudaStream_t stream)
+{
+    if (capturing(stream)) return;
+    std::lock_guard<std::mutex> lock(in_flight_mu);
+    const RelaxedCapture relaxed;
+    if ((!run->resident_done && cudaEventCreateWithFlags(&run->resident_done, cudaEventDisableTiming) != cudaSuccess) ||
+        cudaEventRecord(run->resident_done, stream) != cudaSuccess || cudaGetDevice(&run->resident_device) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    run->resident_stream = stream;
+    if (run->resident_listed) return;
+    run->resident_listed = true;
+    run->resident_next = in_flight;
+    in_flight = run;
+}
+
+void forget_resident(ga_run *run)
+{
+    if (!run->resident_done) return;
+    std::lock_guard<std::mutex> lock(in_flight_mu);
+    for (ga_run **at = &in_flight; *at; at = &(*at)->resident_next)
+        if (*at == run) {
+            *at = run->resident_next;
+            break;
+        }
+    cudaEventDestroy(run->resident_done);
+    run->resident_done = nullptr;
+}
+
+}  // namespace
+
 int step_run(ga_run *run, uint32_t n_gens, cudaStream_t stream, bool shared)
 {
     if (run->cfg.mode != GA_SYNC) return async_step(run, n_gens, stream);
     if (run->generation + n_gens > 0xFFFFFFFFull) return GA_EINVAL;
     // resident launches: one cooperative launch per chunk of the site table
-    bool resident = false;
+    bool resident = false, fills = false;
     ResidentPlan plan = {};
     if (n_gens > 0 && run->resident_mode != GA_RESIDENT_OFF) {
         const bool eligible = resident_eligible(run), dropping = run->drop_island != 0xFFFFFFFFu;
         bool wanted = eligible;
         if (run->resident_mode == GA_RESIDENT_AUTO && !(eligible && dropping))
             wanted = (eligible || (!shared && !dropping && n_gens >= kResidentAutoGens)) && resident_pays(run);
+        fills = wanted && !eligible;
+        if (fills && run->record_bytes == 16u && another_resident(run, stream)) wanted = false;
         resident = wanted && resident_plan(run, plan);
         if (run->resident_mode == GA_RESIDENT_ON && !resident) return GA_EUNSUPPORTED;
     }
@@ -170,6 +254,7 @@ int step_run(ga_run *run, uint32_t n_gens, cudaStream_t stream, bool shared)
                 resident = false;
                 continue;
             }
+            if (fills) note_resident(run, stream);
             run->cur ^= 1;
             run->generation += chunk;
             n_gens -= chunk;
@@ -521,6 +606,7 @@ int ga_destroy(ga_run *run)
     int rc = GA_OK;
     if (run->batch) rc = ga_batch_remove(run->batch, run);
     if (cudaStreamSynchronize(run->stream) != cudaSuccess) rc = GA_ECUDA;
+    ga::forget_resident(run);
     if (run->owns_workspace && cudaFree(run->workspace) != cudaSuccess) rc = GA_ECUDA;
     delete run;
     return rc;

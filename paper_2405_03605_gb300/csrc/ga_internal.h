@@ -43,6 +43,12 @@ struct ga_run {
     uint32_t resident_mode;
     uint32_t resident_wait_us;
     uint32_t drop_island;
+    // recorded behind a resident launch that takes the GPU (ga_api.cu), with its stream and device
+    cudaEvent_t resident_done;
+    cudaStream_t resident_stream;
+    int resident_device;
+    ga_run *resident_next;  // list of runs whose event was not complete when last asked
+    bool resident_listed;
 };
 
 namespace ga {

@@ -33,3 +33,43 @@ def test_runs_at_once(N, rows, cols, S, every, model):
     for r, s in zip(runs, shapes):
         r.sync()
         assert_same(r.snapshot(), streamed(s, 120), N)
+
+
+def test_large_runs_stream_beside_a_resident_one():
+    """A run that takes the whole GPU when it steps resident streams while another such run does on
+    another stream, and steps resident again when that one is done; one captured into a graph neither
+    asks nor is counted."""
+    import torch
+    from paper_2405_03605_gb300 import ga
+    shapes = [RunShape(rows=96, cols=97, seed=7, run_id=i) for i in range(3)]
+    runs = [ga.Run(s, stream=torch.cuda.Stream()) for s in shapes]
+    for r in runs:
+        r.sync()
+    runs[0].step(4000)  # some 10 ms
+    runs[1].step(30)
+    assert runs[0].launches == 3 and runs[1].launches == 2 + 30
+    runs[0].sync()
+    runs[1].step(30)
+    assert runs[1].launches == 2 + 30 + 2
+    runs[1].step(10)  # its own launches do not count
+    assert runs[1].launches == 2 + 30 + 4
+    runs[1].sync()
+    runs[2].step(20)
+    runs[2].sync()
+    graph = torch.cuda.CUDAGraph()
+    before = runs[2].launches
+    runs[0].step(4000)
+    with torch.cuda.graph(graph, stream=runs[2].stream):
+        runs[2].step(20)
+    assert runs[2].launches == before + 2
+    graph.replay()
+    torch.cuda.synchronize()
+    for r in runs:
+        r.sync()
+    assert_same(runs[1].snapshot(), streamed(shapes[1], 70), 32)
+    assert_same(runs[2].snapshot(), streamed(shapes[2], 40), 32)
+    assert_same(runs[0].snapshot(), streamed(shapes[0], 8000), 32)
+    runs[0].step(2000)
+    runs[0].close()  # with its launch in flight
+    runs[1].step(5)
+    runs[1].sync()
