@@ -38,13 +38,10 @@
 // generation.  The population is then undefined; the status is returned by the next ga_sync.
 //
 // What bounds it: small runs the two L2 trips of a migration (32x32 torus of 32-agent islands:
-// 1.15 us per generation), larger ones issue (9,991 islands of 32: 2.65 us per generation; 7.2 us
-// with one ordinary launch each, 4 with dependent ones).  Shapes, us for 250 generations of 9,991
-// islands of 16-byte and 5,893 of 48-byte records: one warp per block 665 and 562, four 707 and
-// 612 (what depends on the block alone stays in uniform registers); 18 to 20 warps on an SM at up
-// to 96 registers against as many as 64 registers allow: 131,000 agents 1.7 and 2.3 us per
-// generation (the bookkeeping of one island takes a quarter of a warp's lanes), 262,000 2.4 and
-// 2.9.
+// 1.10 us per generation), larger ones issue (9,991 islands of 32: 2.50 us per generation; 7.2 us
+// with one ordinary launch each, 4.3 with dependent ones).  One warp per block: what depends on the
+// block alone stays in uniform registers (250 generations of 9,991 islands of 16-byte and 5,893 of
+// 48-byte records: 665 and 562 us, four warps per block 707 and 612).
 #include "ga_device.cuh"
 #include "ga_internal.h"
 #include "ga_island.cuh"
@@ -59,19 +56,19 @@ namespace {
 // Units per warp: as few as keep an SM's warps to a limit, more where they don't fit at once.  An SM
 // has four schedulers, so a generation lengthens where a sixth warp falls to one of them: with one
 // unit to a warp the limit is 20.  Us per generation with one unit to a warp and with two, on
-// either side of it (2,916 and 3,080 islands of 32): float model 2.23 / 2.26 and 2.57 / 2.28, every 4
-// generations 1.31 / 1.56 and 1.59 / 1.56; trait model every 4 0.76 / 0.77 and 0.90 / 0.77.  (A limit of
-// 18 takes two from 2,737 on: 1.55 for the float model every 4, which took 1.41 with a warp to
-// every island.)  But
+// either side of it (2,916 to 3,025 and 3,080 islands of 32): float model 2.08 / 2.20 and 2.34 / 2.20,
+// every 4 generations 1.23 / 1.49 and 1.46 / 1.49; trait model every 4 0.70 / 0.73 and 0.81 / 0.73.
+// (A limit of 18, which takes two from 2,737 on, made the float model slower there than with a warp
+// to every island before: 1.55 against 1.41 every 4.)  But
 //   - float model, and islands of 16, with tournaments of run-time size and several generations to
-//     a migration: a unit's work is long, so one to a warp whatever the registers allow (25 to 28
-//     warps): 3,403 units 1.71 / 1.82 every 4, 1.54 / 1.59 every 16;
+//     a migration: a unit's work is long, so one to a warp up to 28 warps: 3,422 islands of 32 every 4
+//     1.51 / 1.63, every 16 1.38 / 1.42;
 //   - 16-byte trait records in islands of 32 or 64, tournaments of 5, a migration in one or two
 //     generations: so short that from 16 warps on two to a warp are faster, as the bookkeeping of
-//     one fills few of a warp's lanes: 2,500 and 2,704 islands of 32 1.62 / 1.55 and 1.67 / 1.57, of 64
-//     2.23 / 2.04, every 2 1.06 / 1.03.
-// With more units to a warp, 18: 14,062 islands of 32 5 or 6 to a warp (18.5 and 15.4 warps) 3.42 and
-// 3.12, float model 6.14 and 5.75; 48-byte records in islands of 16 6.3 and 5.7.
+//     one fills few of a warp's lanes: 2,401 islands of 32 1.40 / 1.43, 2,601 1.50 / 1.45, 3,025 1.55 /
+//     1.50; 2,652 of 64 2.02 / 1.95.
+// With more units to a warp, 18: 14,042 islands of 32 five or six to a warp (18.5 and 15.4 warps) 3.19
+// and 2.95, float model 5.83 and 5.52.
 uint32_t units_per_warp(const ga_run *run, uint32_t n_units, uint32_t sms)
 {
     const bool five = run->cfg.tournament_size == 5u, fit = run->cfg.model == GA_MODEL_FITNESS;

@@ -73,3 +73,31 @@ def test_large_runs_stream_beside_a_resident_one():
     runs[0].close()  # with its launch in flight
     runs[1].step(5)
     runs[1].sync()
+
+
+def test_runs_of_several_threads():
+    """Handles of their own in threads of their own, large enough to fill the GPU resident."""
+    import threading
+
+    import torch
+    from paper_2405_03605_gb300 import ga
+    shapes = [RunShape(rows=96, cols=98, seed=9, run_id=i) for i in range(4)]
+    runs = [ga.Run(s, stream=torch.cuda.Stream()) for s in shapes]
+    failed = []
+
+    def work(r):
+        try:
+            for _ in range(12):
+                r.step(10)
+                r.sync()
+        except Exception as e:
+            failed.append(e)
+
+    threads = [threading.Thread(target=work, args=(r,)) for r in runs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
+    for r, s in zip(runs, shapes):
+        assert_same(r.snapshot(), streamed(s, 120), 32)
