@@ -557,10 +557,11 @@ bool resident_eligible(const ga_run *run)
 // most agents, in thousands, up to which they are faster; rows: islands of 8, 16, 32, 64; columns:
 // 16-byte trait records, the float model, 32-byte, 48-byte records.  Streamed / resident, us per
 // generation (the slower of tournaments of 5 and 3) on either side of some lines:
-//   k = 1   16-byte: 16: 350 4.3 / 3.6, 400 4.1 / 4.7; 32: 1,000 7.1 / 6.9, 1,100 7.1 / 7.7; 64: 1,100 8.5 / 8.5
-//           float: 32: 750 9.0 / 8.8, 800 9.1 / 10.6;  32-byte: 16: 700 8.94 / 8.93, 1,000 12.0 / 31
+//   k = 1   16-byte: 16: 350 4.1 / 3.2, 400 4.1 / 4.5; 32: 1,000 7.1 / 6.5, 1,100 7.1 / 7.3; 64: 1,100 8.5 / 8.1
+//           float: 32: 650 8.9 / 8.5, 750 9.0 / 10.1;  32-byte: 16: 700 8.94 / 8.93, 1,000 12.0 / 31
 //           48-byte: 16: 650 10.2 / 8.8, 700 10.7 / 28 (too few warps fit); 64: 700 10.4 / 7.5
-//   k = 2   48-byte: 16: 600 5.85 / 5.77, 700 6.5 / 22; 32: 600 5.45 / 4.37;  32-byte: 64: 450 3.9 / 3.9
+//   k = 2   48-byte: 16: 600 5.85 / 5.77, 700 6.5 / 22; 32: 600 5.45 / 4.37;  32-byte: 64: 450 3.9 / 3.9;
+//           float: 64: 900 14.1 / 11.3, 1,100 14.1 / 16.9
 //   k = 4   32-byte: 16: 65 1.00, 98 0.91 of the streamed rate; 32: 98 1.02, 131 0.92; 64: 114 1.05, 131 0.95
 //   k = 6   48-byte: 32: 150 1.02, 175 0.93; 64: 114 0.97 to 1.06, 131 0.89 to 0.98;  k = 8: 32: 65 0.99, 81 0.96
 struct ResidentLines {
@@ -568,8 +569,8 @@ struct ResidentLines {
     uint16_t most[4][4];
 };
 constexpr ResidentLines kResidentLines[] = {
-    {1u, {{150, 0, 0, 150}, {380, 375, 700, 650}, {1000, 750, 1100, 700}, {1400, 1400, 1000, 700}}},
-    {2u, {{99, 0, 0, 99}, {300, 275, 300, 600}, {500, 500, 550, 600}, {1400, 1400, 450, 600}}},
+    {1u, {{150, 0, 0, 150}, {380, 375, 700, 650}, {1000, 650, 1100, 700}, {1400, 1000, 1000, 700}}},
+    {2u, {{99, 0, 0, 99}, {300, 225, 300, 600}, {500, 500, 550, 600}, {1400, 950, 450, 600}}},
     {4u, {{66, 0, 0, 66}, {200, 200, 66, 150}, {400, 400, 99, 200}, {600, 600, 115, 150}}},
     {6u, {{66, 0, 0, 66}, {200, 200, 0, 50}, {400, 400, 50, 150}, {600, 600, 66, 115}}},
     {8u, {{66, 0, 0, 0}, {200, 200, 0, 0}, {400, 400, 0, 66}, {600, 600, 0, 33}}},

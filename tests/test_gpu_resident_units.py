@@ -40,7 +40,7 @@ def test_several_islands_to_a_warp(N, rows, cols, S, every, tsize, model, gens):
 @pytest.mark.parametrize("N,rows,cols,S,every,model,launches", [
     (16, 200, 203, 256, 1, MODEL_TRAIT, 3), (16, 205, 210, 256, 1, MODEL_TRAIT, 2 + 8),
     (16, 290, 210, 128, 1, MODEL_TRAIT, 2 + 8), (16, 64, 65, 128, 4, MODEL_TRAIT, 2 + 2),
-    (32, 150, 151, 64, 1, MODEL_FITNESS, 3), (32, 160, 160, 64, 1, MODEL_FITNESS, 2 + 8),
+    (32, 140, 141, 64, 1, MODEL_FITNESS, 3), (32, 150, 151, 64, 1, MODEL_FITNESS, 2 + 8),
     (64, 25, 41, 128, 8, MODEL_TRAIT, 2 + 1), (8, 110, 110, 256, 1, MODEL_TRAIT, 3),
 ])
 def test_auto_streams_where_that_is_faster(N, rows, cols, S, every, model, launches):
