@@ -45,9 +45,9 @@ def test_large_runs_stream_beside_a_resident_one():
     runs = [ga.Run(s, stream=torch.cuda.Stream()) for s in shapes]
     for r in runs:
         r.sync()
-    runs[0].step(4000)  # some 10 ms
+    runs[0].step(12000)  # some 30 ms
     runs[1].step(30)
-    assert runs[0].launches == 3 and runs[1].launches == 2 + 30
+    assert runs[0].launches == 1 + 3 * 2 and runs[1].launches == 2 + 30
     runs[0].sync()
     runs[1].step(30)
     assert runs[1].launches == 2 + 30 + 2
@@ -68,7 +68,7 @@ def test_large_runs_stream_beside_a_resident_one():
         r.sync()
     assert_same(runs[1].snapshot(), streamed(shapes[1], 70), 32)
     assert_same(runs[2].snapshot(), streamed(shapes[2], 40), 32)
-    assert_same(runs[0].snapshot(), streamed(shapes[0], 8000), 32)
+    assert_same(runs[0].snapshot(), streamed(shapes[0], 16000), 32)
     runs[0].step(2000)
     runs[0].close()  # with its launch in flight
     runs[1].step(5)
